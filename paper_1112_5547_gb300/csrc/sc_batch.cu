@@ -52,7 +52,9 @@ template <class L, class S, int TX, int TY>
 cudaError_t launch_batch(const void* lats, const BatchItem* items, int nitems, int parity, int sm_count, int* ctr,
                          bool grid_mode, cudaStream_t st) {
     using C = typename Codec<S>::C;
-    constexpr int kMin = sizeof(C) == 8 ? 1 : (TX * TY <= 128 ? 4 : 2);
+    // D2Q9: as the solo kernel (step_tiled), more CTAs with fewer registers
+    constexpr int kMin = L::D == 2 ? (sizeof(C) == 8 ? 2 : 3) * (TX * TY <= 128 ? 2 : 1)
+                                   : sizeof(C) == 8 ? 1 : (TX * TY <= 128 ? 4 : 2);
     constexpr auto kern = sc_batch_step_kernel<L, S, TX, TY, kMin>;
     int per_sm = 1;  // resident CTAs per SM
     const cudaError_t oe = blocks_per_sm_once<kern>(TX * TY, &per_sm);

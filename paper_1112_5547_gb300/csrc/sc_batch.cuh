@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     constexpr int NPL = L::D == 3 ? 3 : 1;
     constexpr int H = 2 * FX + 2 * TY;
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
-    __shared__ C srho[NPL][2][FY][FX];
+    __shared__ Two<C> srho[NPL][FY][FX];
     __shared__ int s_next;
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
@@ -89,21 +89,19 @@ __global__ void __launch_bounds__(TX* TY, MINB)
 
         auto density_plane = [&](int slot, int z, C (&f)[2][Q]) {
             pull_node<L, S>(a, gx, gy, z, f);
-            srho[slot][0][ty + 1][tx + 1] = node_density<L, C>(f[0]);
-            srho[slot][1][ty + 1][tx + 1] = node_density<L, C>(f[1]);
+            srho[slot][ty + 1][tx + 1] = node_densities<L, C>(f);
             if (halo) {
                 C h[2][Q];
                 pull_node<L, S>(a, hgx, hgy, z, h);
-                srho[slot][0][hfy][hfx] = node_density<L, C>(h[0]);
-                srho[slot][1][hfy][hfx] = node_density<L, C>(h[1]);
+                srho[slot][hfy][hfx] = node_densities<L, C>(h);
             }
         };
         auto process = [&](C (&f)[2][Q], int sm, int sc, int sp, int z) {
-            const C rA = srho[sc][0][ty + 1][tx + 1];
-            const C rB = srho[sc][1][ty + 1][tx + 1];
-            auto nbr = [&](int s, int i) -> C {
+            const Two<C> r = srho[sc][ty + 1][tx + 1];
+            const C rA = r.a, rB = r.b;
+            auto nbr = [&](int i) -> Two<C> {
                 const int slot = L::c(i, 2) == 0 ? sc : (L::c(i, 2) > 0 ? sp : sm);
-                return srho[slot][s][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
+                return srho[slot][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
             };
             node_update<L, C>(a, gy, nbr, f, rA, rB);
             if (owner) store_node<L, S>(a, gx, gy, z, f, rA, rB);

@@ -224,6 +224,82 @@ template <> struct Ar<double> {
     __device__ __forceinline__ static double rcp(double a) { return __drcp_rn(a); }
 };
 
+// A value of each species (A in a, B in b), and the same operations on both.
+// FP32 uses the packed instructions (FADD2 / FMUL2 / FFMA2: two roundings to
+// nearest in one issue slot), so the pair's results are those of the two
+// scalar operations.  The step kernels issue about half as many arithmetic
+// instructions that way; see node_collide.
+template <class C> struct alignas(2 * sizeof(C)) Two {
+    C a, b;
+};
+template <class C> __device__ __forceinline__ Two<C> both(C v) { return Two<C>{v, v}; }
+template <class C> __device__ __forceinline__ Two<C> neg2(Two<C> v) { return Two<C>{-v.a, -v.b}; }
+__device__ __forceinline__ double neg2(double v) { return -v; }
+__device__ __forceinline__ float neg2(float v) { return -v; }
+template <class C> struct Ar2 {
+    using T = Two<C>;
+    using A = Ar<C>;
+    __device__ __forceinline__ static T add(T x, T y) { return T{A::add(x.a, y.a), A::add(x.b, y.b)}; }
+    __device__ __forceinline__ static T sub(T x, T y) { return T{A::sub(x.a, y.a), A::sub(x.b, y.b)}; }
+    __device__ __forceinline__ static T mul(T x, T y) { return T{A::mul(x.a, y.a), A::mul(x.b, y.b)}; }
+    __device__ __forceinline__ static T mul_split(T x, T y) { return mul(x, y); }
+    __device__ __forceinline__ static T fma(T x, T y, T z) { return T{A::fma(x.a, y.a, z.a), A::fma(x.b, y.b, z.b)}; }
+};
+// A packed product must not meet a packed (or scalar) addition: the assembler
+// contracts the two into one FFMA2 even where both are written with .rn
+// (measured: other last digits than the scalar operations in 39 % of random
+// sums), so products that are added to something use mul_split, two scalar
+// multiplications.  Products that go into a multiplication or are the addend
+// of an fma cannot be contracted.
+template <> struct Ar2<float> {
+    using T = Two<float>;
+    using P = unsigned long long;
+    __device__ __forceinline__ static P in(T x) {
+        P p;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(x.a), "f"(x.b));
+        return p;
+    }
+    __device__ __forceinline__ static T out(P p) {
+        T x;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(x.a), "=f"(x.b) : "l"(p));
+        return x;
+    }
+    __device__ __forceinline__ static T add(T x, T y) {
+        P r;
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(in(x)), "l"(in(y)));
+        return out(r);
+    }
+    __device__ __forceinline__ static T sub(T x, T y) { return add(x, neg2(y)); }
+    __device__ __forceinline__ static T mul(T x, T y) {
+        P r;
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(in(x)), "l"(in(y)));
+        return out(r);
+    }
+    __device__ __forceinline__ static T mul_split(T x, T y) { return T{__fmul_rn(x.a, y.a), __fmul_rn(x.b, y.b)}; }
+    __device__ __forceinline__ static T fma(T x, T y, T z) {
+        P r;
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(in(x)), "l"(in(y)), "l"(in(z)));
+        return out(r);
+    }
+};
+
+// What the relaxation of one node works on at a time, and its operations: both
+// species for FP32 (packed instructions), one species after the other for FP64
+// (no packed form, and the second species' values would only add registers:
+// the FP64 kernels sit at the 255-register limit).
+template <class V> struct Vops;
+template <class C> struct Vops<Two<C>> : Ar2<C> {
+    __device__ __forceinline__ static Two<C> c(C v) { return both(v); }
+};
+template <> struct Vops<float> : Ar<float> {
+    __device__ __forceinline__ static float c(float v) { return v; }
+    __device__ __forceinline__ static float mul_split(float a, float b) { return __fmul_rn(a, b); }
+};
+template <> struct Vops<double> : Ar<double> {
+    __device__ __forceinline__ static double mul_split(double a, double b) { return __dmul_rn(a, b); }
+    __device__ __forceinline__ static double c(double v) { return v; }
+};
+
 // Storage index of cell (x, y, z), x in [-gxo, px - gxo), y in [-gyo, py - gyo).
 template <class Args> __device__ __forceinline__ size_t cell(const Args& a, int x, int y, int z) {
     return (size_t)(x + a.gxo) + (size_t)a.px * ((size_t)(y + a.gyo) + (size_t)a.py * (size_t)z);

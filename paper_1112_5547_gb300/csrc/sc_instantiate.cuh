@@ -15,8 +15,12 @@ template <class L, class S, int TX, int TY>
 cudaError_t step_tiled(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) {
     using C = typename Codec<S>::C;
     FieldArgs<C> fo{};
-    // register budget: 65536 / (threads * CTAs per SM)
-    constexpr int kMin = sizeof(C) == 8 ? 1 : (TX * TY <= 128 ? 4 : (TX * TY <= 256 ? 2 : 1));
+    // register budget: 65536 / (threads * CTAs per SM).  A D2Q9 CTA holds one
+    // row block and no pipeline, so its loads in flight are its warps': three
+    // CTAs of 256 threads (80 registers) rather than two (90), 0.50 against
+    // 0.67 ms a step at 4096^2; two (128 registers) in FP64.
+    constexpr int kMin = L::D == 2 ? (sizeof(C) == 8 ? 2 : 3) * (TX * TY <= 128 ? 2 : 1) / (TX * TY > 256 ? 2 : 1)
+                         : sizeof(C) == 8 ? 1 : (TX * TY <= 128 ? 4 : (TX * TY <= 256 ? 2 : 1));
     sc_fused_kernel<L, S, TX, TY, kModeStep, kMin><<<step_grid(p), dim3(TX, TY), 0, st>>>(a, fo);
     return cudaGetLastError();
 }

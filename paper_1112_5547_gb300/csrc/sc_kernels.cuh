@@ -105,6 +105,22 @@ __device__ __forceinline__ void store_node(const LatticeArgs<S>& a, int x, int y
     // write (measured: 20 % more write traffic on 128-wide rows without it)
     constexpr int kSector = 32 / (int)sizeof(S) > 2 ? 32 / (int)sizeof(S) : 2;
     const int GX = nx >= kSector ? kSector : 2;
+    if (nx >= 2 * kSector && ny >= 4) {
+        // a node has at most one image along x, one along y and the corner of
+        // both: their offsets are formed directly (a walk over all 24 image
+        // offsets of a tiny lattice, below, costs the warps at the edges of a
+        // tile about as many instructions again as their collision)
+        const int ox = x < GX ? nx : (x >= nx - GX ? -nx : 0);
+        const int oy = y < 2 ? ny : (y >= ny - 2 ? -ny : 0);
+        if ((ox | oy) != 0) {
+#pragma unroll 1
+            for (int k = 1; k < 4; ++k) {
+                if (((k & 1) && ox == 0) || ((k & 2) && oy == 0)) continue;
+                store_cell<L, S>(a, cell(a, x + ((k & 1) ? ox : 0), y + ((k & 2) ? oy : 0), z), f, base);
+            }
+        }
+        return;
+    }
     if (x < GX || x >= nx - GX || y < 2 || y >= ny - 2) {
 #pragma unroll 1
         for (int ix = -2; ix <= 2; ++ix) {
@@ -153,7 +169,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     constexpr int NPL = L::D == 3 ? 3 : 1;
     constexpr int H = 2 * FX + 2 * TY;
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
-    __shared__ C srho[NPL][2][FY][FX];
+    __shared__ Two<C> srho[NPL][FY][FX];  // densities (rho_A, rho_B)
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -176,22 +192,20 @@ __global__ void __launch_bounds__(TX* TY, MINB)
 
     auto density_plane = [&](int slot, int z, C (&f)[2][Q]) {
         pull_node<L, S>(a, gx, gy, z, f);
-        srho[slot][0][ty + 1][tx + 1] = node_density<L, C>(f[0]);
-        srho[slot][1][ty + 1][tx + 1] = node_density<L, C>(f[1]);
+        srho[slot][ty + 1][tx + 1] = node_densities<L, C>(f);
         if (halo) {
             C h[2][Q];
             pull_node<L, S>(a, hgx, hgy, z, h);
-            srho[slot][0][hfy][hfx] = node_density<L, C>(h[0]);
-            srho[slot][1][hfy][hfx] = node_density<L, C>(h[1]);
+            srho[slot][hfy][hfx] = node_densities<L, C>(h);
         }
     };
 
     auto process = [&](C (&f)[2][Q], int sm, int sc, int sp, int z) {
-        const C r0 = srho[sc][0][ty + 1][tx + 1];
-        const C r1 = srho[sc][1][ty + 1][tx + 1];
-        auto nbr = [&](int s, int i) -> C {
+        const Two<C> r01 = srho[sc][ty + 1][tx + 1];
+        const C r0 = r01.a, r1 = r01.b;
+        auto nbr = [&](int i) -> Two<C> {
             const int slot = L::c(i, 2) == 0 ? sc : (L::c(i, 2) > 0 ? sp : sm);
-            return srho[slot][s][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
+            return srho[slot][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
         };
         const size_t node = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * z);
         if (MODE == kModeStep) {
@@ -209,16 +223,15 @@ __global__ void __launch_bounds__(TX* TY, MINB)
             }
             const C rA = fe ? A::mul((C)0.5, A::add(r0, r1)) : r0;
             const C rB = fe ? A::mul((C)0.5, A::sub(r0, r1)) : r1;
-            C jA[3], jB[3] = {(C)0, (C)0, (C)0};
-            node_momentum<L, C>(f[0], jA);
-            if (!fe) node_momentum<L, C>(f[1], jB);
+            Two<C> j[3];
+            node_momenta<L, C>(f, j);
             const C rho = fe ? r0 : A::add(rA, rB);
             const C inv_rho = A::rcp(rho);
             C u[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 const C half_force = A::mul((C)0.5, A::fma(rA, gA[d], A::mul(rB, gB[d])));
-                u[d] = A::mul(A::add(A::add(jA[d], jB[d]), half_force), inv_rho);
+                u[d] = A::mul(A::add(fe ? j[d].a : A::add(j[d].a, j[d].b), half_force), inv_rho);
             }
             const C p = A::mul(A::fma(A::mul(a.G, rA), rB, rho), (C)(1.0 / 3.0));
             if (owner) {
@@ -340,7 +353,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
     constexpr int NPL = L::D == 3 ? 4 : 1;
     constexpr int H = 2 * FX + 2 * TY;
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
-    __shared__ C ring[NPL][2][FY][FX];
+    __shared__ Two<C> ring[NPL][FY][FX];
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -356,22 +369,20 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
     auto density_plane = [&](int slot, int z) {
         C f[2][Q];
         pull_node<L, S>(a, gx, gy, z, f);
-        ring[slot][0][ty + 1][tx + 1] = node_density<L, C>(f[0]);
-        ring[slot][1][ty + 1][tx + 1] = node_density<L, C>(f[1]);
+        ring[slot][ty + 1][tx + 1] = node_densities<L, C>(f);
         if (halo) {
             pull_node<L, S>(a, hgx, hgy, z, f);
-            ring[slot][0][hfy][hfx] = node_density<L, C>(f[0]);
-            ring[slot][1][hfy][hfx] = node_density<L, C>(f[1]);
+            ring[slot][hfy][hfx] = node_densities<L, C>(f);
         }
     };
     auto collide = [&](int sm, int sc, int sp, int z) {
         C f[2][Q];
         pull_node<L, S>(a, gx, gy, z, f);
-        const C rA = ring[sc][0][ty + 1][tx + 1];
-        const C rB = ring[sc][1][ty + 1][tx + 1];
-        auto nbr = [&](int s, int i) -> C {
+        const Two<C> r = ring[sc][ty + 1][tx + 1];
+        const C rA = r.a, rB = r.b;
+        auto nbr = [&](int i) -> Two<C> {
             const int sl = L::c(i, 2) == 0 ? sc : (L::c(i, 2) > 0 ? sp : sm);
-            return ring[sl][s][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
+            return ring[sl][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
         };
         node_update<L, C>(a, gy, nbr, f, rA, rB);
         if (owner) store_node<L, S>(a, gx, gy, z, f, rA, rB);

@@ -46,6 +46,14 @@ template <class L, class C> __device__ __forceinline__ C node_density(const C (&
     return Ar<C>::add(r, f[0]);
 }
 
+// The densities of both species, each summed as node_density sums it.
+template <class L, class C> __device__ __forceinline__ Two<C> node_densities(const C (&f)[2][L::Q]) {
+    Two<C> r{f[0][1], f[1][1]};
+#pragma unroll
+    for (int i = 2; i < L::Q; ++i) r = Ar2<C>::add(r, Two<C>{f[0][i], f[1][i]});
+    return Ar2<C>::add(r, Two<C>{f[0][0], f[1][0]});
+}
+
 template <class L> __host__ __device__ constexpr bool opposite_pairs() {
     for (int i = 1; i + 1 < L::Q; i += 2)
         for (int d = 0; d < 3; ++d)
@@ -70,6 +78,25 @@ template <class C> struct SignedSum {
     __device__ __forceinline__ C get() const { return empty ? (C)0 : v; }
 };
 
+// The same for a Two or an FP64 value (Vops).
+template <class V> struct SignedSumV {
+    V v;
+    bool empty = true;
+    __device__ __forceinline__ void add(V x) {
+        v = empty ? x : Vops<V>::add(v, x);
+        empty = false;
+    }
+    __device__ __forceinline__ void sub(V x) {
+        v = empty ? neg2(x) : Vops<V>::sub(v, x);
+        empty = false;
+    }
+    __device__ __forceinline__ V get() const {
+        if (!empty) return v;
+        return Vops<V>::c(0);
+    }
+};
+
+// Momentum of one species, and of both.
 template <class L, class C> __device__ __forceinline__ void node_momentum(const C (&f)[L::Q], C (&j)[3]) {
     static_assert(opposite_pairs<L>(), "velocity order must pair c_{i+1} = -c_i");
     SignedSum<C> acc[3];
@@ -86,35 +113,44 @@ template <class L, class C> __device__ __forceinline__ void node_momentum(const 
     for (int d = 0; d < 3; ++d) j[d] = acc[d].get();
 }
 
-// g_s = -G sum_i w_i rho_s'(x + c_i) c_i for both species; nbr(s, i) returns
-// rho_s(x + c_i).
+template <class L, class C> __device__ __forceinline__ void node_momenta(const C (&f)[2][L::Q], Two<C> (&j)[3]) {
+    static_assert(opposite_pairs<L>(), "velocity order must pair c_{i+1} = -c_i");
+    SignedSumV<Two<C>> acc[3];
+#pragma unroll
+    for (int i = 1; i < L::Q; i += 2) {
+        const Two<C> dlt = Ar2<C>::sub(Two<C>{f[0][i], f[1][i]}, Two<C>{f[0][i + 1], f[1][i + 1]});
+#pragma unroll
+        for (int d = 0; d < L::D; ++d) {
+            if (L::c(i, d) == 1) acc[d].add(dlt);
+            if (L::c(i, d) == -1) acc[d].sub(dlt);
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) j[d] = acc[d].get();
+}
+
+// g_s = -G sum_i w_i rho_s'(x + c_i) c_i for both species; nbr(i) returns the
+// pair (rho_A, rho_B) at x + c_i.
 template <class L, class C, class Nbr>
 __device__ __forceinline__ void node_force(const Nbr& nbr, C G, C (&gA)[3], C (&gB)[3]) {
-    using A = Ar<C>;
+    using A2 = Ar2<C>;
     static_assert(opposite_pairs<L>(), "velocity order must pair c_{i+1} = -c_i");
-    gA[0] = gA[1] = gA[2] = gB[0] = gB[1] = gB[2] = (C)0;
+    Two<C> g[3] = {both((C)0), both((C)0), both((C)0)};  // (g_B, g_A) / -G: each species feels the other's density
 #pragma unroll
     for (int i = 1; i < L::Q; i += 2) {
         const C w = (C)L::w(i);
-        const C dA = A::sub(nbr(0, i), nbr(0, i + 1));  // rho_A(x + c_i) - rho_A(x - c_i)
-        const C dB = A::sub(nbr(1, i), nbr(1, i + 1));
+        const Two<C> dr = A2::sub(nbr(i), nbr(i + 1));  // rho(x + c_i) - rho(x - c_i)
 #pragma unroll
         for (int d = 0; d < L::D; ++d) {
-            if (L::c(i, d) == 1) {
-                gA[d] = A::fma(w, dB, gA[d]);
-                gB[d] = A::fma(w, dA, gB[d]);
-            }
-            if (L::c(i, d) == -1) {
-                gA[d] = A::fma(-w, dB, gA[d]);
-                gB[d] = A::fma(-w, dA, gB[d]);
-            }
+            if (L::c(i, d) == 1) g[d] = A2::fma(both(w), dr, g[d]);
+            if (L::c(i, d) == -1) g[d] = A2::fma(both(-w), dr, g[d]);
         }
     }
-    const C mG = -G;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        gA[d] = A::mul(gA[d], mG);
-        gB[d] = A::mul(gB[d], mG);
+        const Two<C> h = A2::mul_split(g[d], both(-G));
+        gA[d] = h.b;
+        gB[d] = h.a;
     }
 }
 
@@ -159,45 +195,97 @@ template <class L, class C> __device__ __forceinline__ C node_cu(int i, const C 
     return cu.get();
 }
 
-// BGK relaxation of one species towards f^eq(rho, u), each moving population
-// relaxed as soon as its equilibrium is formed (fewer live values), the rest
-// population last from the closure f^eq_0 = rho - sum_{i>0} f^eq_i, taken as
+template <class L, class V> __device__ __forceinline__ V node_cu2(int i, const V (&u)[3]) {
+    SignedSumV<V> cu;
+#pragma unroll
+    for (int d = 0; d < L::D; ++d) {
+        if (L::c(i, d) == 1) cu.add(u[d]);
+        if (L::c(i, d) == -1) cu.sub(u[d]);
+    }
+    return cu.get();
+}
+
+// a.b of two vectors, summed from the last component down.
+template <class L, class V> __device__ __forceinline__ V node_dot2(const V (&a)[3], const V (&b)[3]) {
+    using A = Vops<V>;
+    return L::D == 3 ? A::fma(a[0], b[0], A::fma(a[1], b[1], A::mul(a[2], b[2]))) : A::fma(a[0], b[0], A::mul(a[1], b[1]));
+}
+
+// The populations the relaxation works on: both species of a node, or one.
+template <class L, class C> struct BothF {
+    using V = Two<C>;
+    C (&f)[2][L::Q];
+    __device__ __forceinline__ V get(int i) const { return V{f[0][i], f[1][i]}; }
+    __device__ __forceinline__ void set(int i, V v) const {
+        f[0][i] = v.a;
+        f[1][i] = v.b;
+    }
+};
+template <class L, class C> struct OneF {
+    using V = C;
+    C (&f)[L::Q];
+    __device__ __forceinline__ V get(int i) const { return f[i]; }
+    __device__ __forceinline__ void set(int i, V v) const { f[i] = v; }
+};
+
+// BGK relaxation towards f^eq(rho_s, u_s), each moving population relaxed as
+// soon as its equilibrium is formed (fewer live values), the rest population
+// last from the closure f^eq_0 = rho - sum_{i>0} f^eq_i, taken as
 // f^eq_0 - f_0 = -sum_{i>0} (f^eq_i - f_i).
-template <class L, class C> __device__ __forceinline__ void node_relax(C (&f)[L::Q], C rho, const C (&u)[3], C omega) {
-    using A = Ar<C>;
-    C uu = L::D == 3 ? A::fma(u[0], u[0], A::fma(u[1], u[1], A::mul(u[2], u[2]))) : A::fma(u[0], u[0], A::mul(u[1], u[1]));
-    const C base = A::fma((C)-1.5, uu, (C)1);
-    SignedSum<C> neq;  // sum_{i>0} (f^eq_i - f_i)
+template <class L, class F, class V = typename F::V>
+__device__ __forceinline__ void node_relax(const F& f, V rho, const V (&u)[3], V omega) {
+    using A = Vops<V>;
+    const V base = A::fma(A::c(-1.5), node_dot2<L, V>(u, u), A::c(1));
+    SignedSumV<V> neq;  // sum_{i>0} (f^eq_i - f_i)
 #pragma unroll
     for (int i = 1; i < L::Q; ++i) {
-        const C cu = node_cu<L, C>(i, u);
-        const C wr = A::mul((C)L::w(i), rho);
-        const C feq = A::mul(wr, A::fma(cu, A::fma((C)4.5, cu, (C)3), base));
-        const C d = A::sub(feq, f[i]);
+        const V cu = node_cu2<L, V>(i, u);
+        const V wr = A::mul(A::c(L::w(i)), rho);
+        const V feq = A::mul_split(wr, A::fma(cu, A::fma(A::c(4.5), cu, A::c(3)), base));
+        const V d = A::sub(feq, f.get(i));
         neq.add(d);
-        f[i] = A::fma(omega, d, f[i]);
+        f.set(i, A::fma(omega, d, f.get(i)));
     }
-    f[0] = A::fma(omega, -neq.get(), f[0]);  // f^eq_0 - f_0 = -sum_{i>0} (f^eq_i - f_i)
+    f.set(0, A::fma(omega, neg2(neq.get()), f.get(0)));
+}
+
+// Component s of a pair of vectors.
+template <class C> __device__ __forceinline__ void node_part(const Two<C> (&v)[3], int s, C (&o)[3]) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) o[d] = s == 0 ? v[d].a : v[d].b;
 }
 
 // Collision of both species of one node: common velocity shifted by tau_s g_s.
-template <class L, class C>
+// PACK: both species relax together in the packed FP32 instructions, which
+// halves the arithmetic instructions of a step (a TMA-fed step is bound by
+// issue and by its per-plane barrier as much as by HBM; measured with the
+// direct ghost images of store_node: 512^3 FP32 7.66 -> 7.13 ms, 256^3 1.05 ->
+// 0.975, Guo forcing at 128^3 0.207 -> 0.180).  The kernels that hold two CTAs
+// of 256 threads per SM have 128 registers a thread: the pairs (and their
+// constants) then spill, so they relax one species after the other and keep
+// only the sums packed (512^3 bf16 rest-offset 5.52 ms packed with 84 bytes of
+// spills, 5.28 so, 5.46 before).
+template <class L, class C, bool PACK = sizeof(C) == 4>
 __device__ __forceinline__ void node_collide(C (&f)[2][L::Q], C rA, C rB, const C (&gA)[3], const C (&gB)[3],
                                              C omega_A, C omega_B, C tau_A, C tau_B) {
     using A = Ar<C>;
-    C jA[3], jB[3];
-    node_momentum<L, C>(f[0], jA);
-    node_momentum<L, C>(f[1], jB);
+    Two<C> j[3], u[3];
+    node_momenta<L, C>(f, j);
     const C inv_den = A::rcp(A::fma(rA, omega_A, A::mul(rB, omega_B)));
-    C uA[3], uB[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const C up = A::mul(A::fma(jA[d], omega_A, A::mul(jB[d], omega_B)), inv_den);
-        uA[d] = A::fma(tau_A, gA[d], up);
-        uB[d] = A::fma(tau_B, gB[d], up);
+        const C up = A::mul(A::fma(j[d].a, omega_A, A::mul(j[d].b, omega_B)), inv_den);
+        u[d] = Ar2<C>::fma(Two<C>{tau_A, tau_B}, Two<C>{gA[d], gB[d]}, both(up));
     }
-    node_relax<L, C>(f[0], rA, uA, omega_A);
-    node_relax<L, C>(f[1], rB, uB, omega_B);
+    if constexpr (PACK) {
+        node_relax<L>(BothF<L, C>{f}, Two<C>{rA, rB}, u, Two<C>{omega_A, omega_B});
+    } else {
+        C us[3];
+        node_part<C>(u, 0, us);
+        node_relax<L>(OneF<L, C>{f[0]}, rA, us, omega_A);
+        node_part<C>(u, 1, us);
+        node_relax<L>(OneF<L, C>{f[1]}, rB, us, omega_B);
+    }
 }
 
 // Guo forcing, the discrete-forcing cure that Sec. 2.3 names for the
@@ -210,60 +298,62 @@ __device__ __forceinline__ void node_collide(C (&f)[2][L::Q], C rA, C rB, const 
 // i vanishes in exact arithmetic), and f^eq_0 as in node_relax.  Opposite directions share
 // their terms: with t1 = 9 (c.u)(c.F) - 3 u.F and t2 = 3 c.F (c = c_i),
 // S_i = w_i (t1 + t2) and S_{i+1} = w_i (t1 - t2), since c_{i+1} = -c_i.
-template <class L, class C>
-__device__ __forceinline__ void node_relax_guo(C (&f)[L::Q], C rho, const C (&u)[3], const C (&F)[3], C omega) {
-    using A = Ar<C>;
-    C uu = L::D == 3 ? A::fma(u[0], u[0], A::fma(u[1], u[1], A::mul(u[2], u[2]))) : A::fma(u[0], u[0], A::mul(u[1], u[1]));
-    C uF = L::D == 3 ? A::fma(u[0], F[0], A::fma(u[1], F[1], A::mul(u[2], F[2]))) : A::fma(u[0], F[0], A::mul(u[1], F[1]));
-    const C base = A::fma((C)-1.5, uu, (C)1);
-    const C keep = A::fma((C)-0.5, omega, (C)1);  // 1 - 1 / (2 tau)
-    const C m3uF = A::mul((C)-3, uF);
+template <class L, class F, class V = typename F::V>
+__device__ __forceinline__ void node_relax_guo(const F& f, V rho, const V (&u)[3], const V (&force)[3], V omega) {
+    using A = Vops<V>;
+    const V base = A::fma(A::c(-1.5), node_dot2<L, V>(u, u), A::c(1));
+    const V keep = A::fma(A::c(-0.5), omega, A::c(1));  // 1 - 1 / (2 tau)
+    const V m3uF = A::mul(A::c(-3), node_dot2<L, V>(u, force));
     static_assert(opposite_pairs<L>(), "velocity order must pair c_{i+1} = -c_i");
-    SignedSum<C> neq, sources;
+    SignedSumV<V> neq, sources;
 #pragma unroll
     for (int i = 1; i < L::Q; i += 2) {
-        const C cu = node_cu<L, C>(i, u);  // c_{i+1}.u = -cu exactly (a signed sum of the same terms)
-        const C cF = node_cu<L, C>(i, F);
-        const C w = (C)L::w(i);
-        const C wr = A::mul(w, rho);
-        const C feq_p = A::mul(wr, A::fma(cu, A::fma((C)4.5, cu, (C)3), base));
-        const C feq_m = A::mul(wr, A::fma(-cu, A::fma((C)4.5, -cu, (C)3), base));
-        const C d_p = A::sub(feq_p, f[i]);
-        const C d_m = A::sub(feq_m, f[i + 1]);
+        const V cu = node_cu2<L, V>(i, u);  // c_{i+1}.u = -cu exactly (a signed sum of the same terms)
+        const V cF = node_cu2<L, V>(i, force);
+        const V w = A::c(L::w(i)), ncu = neg2(cu);
+        const V wr = A::mul(w, rho);
+        const V feq_p = A::mul_split(wr, A::fma(cu, A::fma(A::c(4.5), cu, A::c(3)), base));
+        const V feq_m = A::mul_split(wr, A::fma(ncu, A::fma(A::c(4.5), ncu, A::c(3)), base));
+        const V d_p = A::sub(feq_p, f.get(i));
+        const V d_m = A::sub(feq_m, f.get(i + 1));
         neq.add(d_p);
         neq.add(d_m);
-        const C t1 = A::fma(A::mul((C)9, cu), cF, m3uF);
-        const C t2 = A::mul((C)3, cF);
-        const C src_p = A::mul(w, A::add(t1, t2));
-        const C src_m = A::mul(w, A::sub(t1, t2));
+        const V t1 = A::fma(A::mul(A::c(9), cu), cF, m3uF);
+        const V t2 = A::mul_split(A::c(3), cF);
+        const V src_p = A::mul_split(w, A::add(t1, t2));
+        const V src_m = A::mul_split(w, A::sub(t1, t2));
         sources.add(src_p);
         sources.add(src_m);
-        f[i] = A::fma(keep, src_p, A::fma(omega, d_p, f[i]));
-        f[i + 1] = A::fma(keep, src_m, A::fma(omega, d_m, f[i + 1]));
+        f.set(i, A::fma(keep, src_p, A::fma(omega, d_p, f.get(i))));
+        f.set(i + 1, A::fma(keep, src_m, A::fma(omega, d_m, f.get(i + 1))));
     }
-    const C src0 = -sources.get();
-    f[0] = A::fma(keep, src0, A::fma(omega, -neq.get(), f[0]));
+    f.set(0, A::fma(keep, neg2(sources.get()), A::fma(omega, neg2(neq.get()), f.get(0))));
 }
 
 template <class L, class C>
 __device__ __forceinline__ void node_collide_guo(C (&f)[2][L::Q], C rA, C rB, const C (&gA)[3], const C (&gB)[3],
                                                  C omega_A, C omega_B) {
     using A = Ar<C>;
-    C jA[3], jB[3];
-    node_momentum<L, C>(f[0], jA);
-    node_momentum<L, C>(f[1], jB);
+    const Two<C> rho{rA, rB};
+    Two<C> j[3], F[3], u[3];
+    node_momenta<L, C>(f, j);
     const C inv_den = A::rcp(A::fma(rA, omega_A, A::mul(rB, omega_B)));
-    C FA[3], FB[3], u[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        FA[d] = A::mul(rA, gA[d]);
-        FB[d] = A::mul(rB, gB[d]);
-        const C mA = A::fma((C)0.5, FA[d], jA[d]);
-        const C mB = A::fma((C)0.5, FB[d], jB[d]);
-        u[d] = A::mul(A::fma(mA, omega_A, A::mul(mB, omega_B)), inv_den);
+        F[d] = Ar2<C>::mul(rho, Two<C>{gA[d], gB[d]});
+        const Two<C> m = Ar2<C>::fma(both((C)0.5), F[d], j[d]);
+        u[d] = both(A::mul(A::fma(m.a, omega_A, A::mul(m.b, omega_B)), inv_den));
     }
-    node_relax_guo<L, C>(f[0], rA, u, FA, omega_A);
-    node_relax_guo<L, C>(f[1], rB, u, FB, omega_B);
+    if constexpr (sizeof(C) == 4) {
+        node_relax_guo<L>(BothF<L, C>{f}, rho, u, F, Two<C>{omega_A, omega_B});
+    } else {
+        C us[3], Fs[3];
+        node_part<C>(u, 0, us);
+        node_part<C>(F, 0, Fs);
+        node_relax_guo<L>(OneF<L, C>{f[0]}, rA, us, Fs, omega_A);
+        node_part<C>(F, 1, Fs);
+        node_relax_guo<L>(OneF<L, C>{f[1]}, rB, us, Fs, omega_B);
+    }
 }
 
 // ---- Free-energy (FE) two-population model (Sec. 2.2) ----------------------
@@ -272,7 +362,7 @@ __device__ __forceinline__ void node_collide_guo(C (&f)[2][L::Q], C rA, C rB, co
 // free energy is the Eq. FEtau functional with coupling g and gradient
 // coefficient kappa; its derivatives come from the isotropic lattice stencils
 //   grad phi = 3 sum_i w_i c_i phi(x + c_i),  lap phi = 6 sum_i w_i (phi(x + c_i) - phi(x)),
-// formed over opposite pairs like the SC force.  nbr(1, i) = phi(x + c_i).
+// formed over opposite pairs like the SC force.  nbr(i).b = phi(x + c_i).
 template <class L, class C, class Nbr>
 __device__ __forceinline__ void node_fe_derivs(const Nbr& nbr, C phi0, C (&gp)[3], C& lp) {
     using A = Ar<C>;
@@ -283,7 +373,7 @@ __device__ __forceinline__ void node_fe_derivs(const Nbr& nbr, C phi0, C (&gp)[3
 #pragma unroll
     for (int i = 1; i < L::Q; i += 2) {
         const C w = (C)L::w(i);
-        const C p = nbr(1, i), m = nbr(1, i + 1);
+        const C p = nbr(i).b, m = nbr(i + 1).b;
         const C d = A::sub(p, m);  // phi(x + c_i) - phi(x - c_i)
 #pragma unroll
         for (int k = 0; k < L::D; ++k) {
@@ -335,31 +425,37 @@ __device__ __forceinline__ void node_collide_fe(C (&f)[2][L::Q], C rho, C phi, c
                        A::mul(cs2, rho));
     const C sg = A::sub(A::mul(gamma, mu), A::mul(cs2, phi));
     const C ku = A::mul(cs2, uu), kg = A::mul(cs2, gg);
-    SignedSum<C> fneq, gneq;  // sum_{i>0} (f^eq_i - f_i), sum_{i>0} (g^eq_i - g_i)
+    // f and g together from here on (first and second of each pair)
+    using A2 = Ar2<C>;
+    const Two<C> rp{rho, phi}, rp3 = A2::mul(both((C)3), rp), om{omega, omega_g}, ss{s, sg}, ku2 = both(ku);
+    Two<C> u2[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) u2[d] = both(u[d]);
+    SignedSumV<Two<C>> neq;  // sum_{i>0} (f^eq_i - f_i), sum_{i>0} (g^eq_i - g_i)
 #pragma unroll
     for (int i = 1; i < L::Q; ++i) {
-        const C cu = node_cu<L, C>(i, u);
+        const Two<C> cu = node_cu2<L>(i, u2);
         const C cg = node_cu<L, C>(i, gp);
         int c2 = 0;
 #pragma unroll
         for (int d = 0; d < L::D; ++d) c2 += L::c(i, d) * L::c(i, d);
         const C iso = (C)((double)c2 - (double)L::D / 3.0);  // c.c - D cs2
-        const C quad_u = A::sub(A::mul(cu, cu), ku);       // (c.u)^2 - cs2 u.u
+        const Two<C> quad_u = A2::sub(A2::mul_split(cu, cu), ku2);  // (c.u)^2 - cs2 u.u
         const C quad_g = A::sub(A::mul(cg, cg), kg);
-        const C w = (C)L::w(i);
-        const C hf = A::fma(s, iso, A::fma(kappa, quad_g, A::mul(rho, quad_u)));
-        const C feq = A::mul(w, A::fma((C)4.5, hf, A::fma(A::mul((C)3, rho), cu, rho)));
-        const C hg = A::fma(sg, iso, A::mul(phi, quad_u));
-        const C geq = A::mul(w, A::fma((C)4.5, hg, A::fma(A::mul((C)3, phi), cu, phi)));
-        const C df = A::sub(feq, f[0][i]);
-        const C dg = A::sub(geq, f[1][i]);
-        fneq.add(df);
-        gneq.add(dg);
-        f[0][i] = A::fma(omega, df, f[0][i]);
-        f[1][i] = A::fma(omega_g, dg, f[1][i]);
+        Two<C> h = A2::mul(rp, quad_u);
+        h.a = A::fma(kappa, quad_g, h.a);
+        h = A2::fma(ss, both(iso), h);
+        const Two<C> feq = A2::mul_split(both((C)L::w(i)), A2::fma(both((C)4.5), h, A2::fma(rp3, cu, rp)));
+        const Two<C> fi{f[0][i], f[1][i]};
+        const Two<C> d = A2::sub(feq, fi);
+        neq.add(d);
+        const Two<C> n = A2::fma(om, d, fi);
+        f[0][i] = n.a;
+        f[1][i] = n.b;
     }
-    f[0][0] = A::fma(omega, -fneq.get(), f[0][0]);
-    f[1][0] = A::fma(omega_g, -gneq.get(), f[1][0]);
+    const Two<C> n = A2::fma(om, neg2(neq.get()), Two<C>{f[0][0], f[1][0]});
+    f[0][0] = n.a;
+    f[1][0] = n.b;
 }
 
 // The collision of the lattice's forcing scheme, chosen at run time (kernels
@@ -376,7 +472,7 @@ __device__ __forceinline__ void node_collide_any(int forcing, C (&f)[2][L::Q], C
 // The whole node update after the pulls: the SC force (and body force) with
 // the lattice's forcing scheme, or the FE derivatives and collision, chosen at
 // run time.  r0, r1: the two population sums of the node (rho_A, rho_B for SC;
-// rho, phi for FE); nbr(s, i) returns the neighbour's sum s at x + c_i.
+// rho, phi for FE); nbr(i) returns the neighbour's pair of sums at x + c_i.
 template <class L, class C, class Args, class Nbr>
 __device__ __forceinline__ void node_update(const Args& a, int y, const Nbr& nbr, C (&f)[2][L::Q], C r0, C r1) {
     if (a.model == kModelFE) {

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_regpipe_kernel(const Lat
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
 
     __shared__ __align__(16) W hst[Q2][H];
-    __shared__ C ring[4][2][FY][FX];
+    __shared__ Two<C> ring[4][FY][FX];
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -110,8 +110,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_regpipe_kernel(const Lat
         pull_node<L, S>(a, gx, gy, z, X);
     };
     auto reduce = [&](int q, const C (&X)[2][Q]) {
-        ring[q & 3][0][ty + 1][tx + 1] = node_density<L, C>(X[0]);
-        ring[q & 3][1][ty + 1][tx + 1] = node_density<L, C>(X[1]);
+        ring[q & 3][ty + 1][tx + 1] = node_densities<L, C>(X);
         cp_async_wait<0>();
         if (halo) {
             C h[2][Q];
@@ -135,17 +134,16 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_regpipe_kernel(const Lat
                         h[s][i] = Codec<S>::decode(v, off);
                     }
                 }
-            ring[q & 3][0][hfy][hfx] = node_density<L, C>(h[0]);
-            ring[q & 3][1][hfy][hfx] = node_density<L, C>(h[1]);
+            ring[q & 3][hfy][hfx] = node_densities<L, C>(h);
         }
     };
     auto collide = [&](int q, C (&X)[2][Q]) {
         const int sm = (q - 1) & 3, sc = q & 3, sp = (q + 1) & 3;
-        const C rA = ring[sc][0][ty + 1][tx + 1];
-        const C rB = ring[sc][1][ty + 1][tx + 1];
-        auto nbr = [&](int s, int i) -> C {
+        const Two<C> r = ring[sc][ty + 1][tx + 1];
+        const C rA = r.a, rB = r.b;
+        auto nbr = [&](int i) -> Two<C> {
             const int sl = L::c(i, 2) == 0 ? sc : (L::c(i, 2) > 0 ? sp : sm);
-            return ring[sl][s][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
+            return ring[sl][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
         };
         C gA[3], gB[3];
         node_force<L, C>(nbr, a.G, gA, gB);

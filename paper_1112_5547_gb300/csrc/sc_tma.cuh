@@ -113,13 +113,13 @@ struct TmaMaps {
 template <int TX, int TY, int S, class St = float> struct TmaSmem {
     using T = TmaTile<TX, TY, S, St>;
     unsigned char* stage;
-    float (*ring)[2][T::FY][T::FX];
+    Two<float> (*ring)[T::FY][T::FX];  // densities (rho_A, rho_B) of four planes
     uint64_t* bars;
 
     __device__ __forceinline__ explicit TmaSmem(unsigned char* raw) {
         unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~(uintptr_t)127);
         stage = base;
-        ring = reinterpret_cast<float(*)[2][T::FY][T::FX]>(base + (size_t)S * T::stage_bytes);
+        ring = reinterpret_cast<Two<float>(*)[T::FY][T::FX]>(base + (size_t)S * T::stage_bytes);
         bars = reinterpret_cast<uint64_t*>(base + (size_t)S * T::stage_bytes + T::ring_bytes);
     }
     __device__ __forceinline__ void init_barriers() {
@@ -357,27 +357,25 @@ __device__ __forceinline__ int tma_item(const CUtensorMap* pmap, const CUtensorM
     auto take_plane = [&](int q, C (&X)[2][Q]) {
         const unsigned char* sb = sm.stage + (size_t)((qbase + q) % S) * T::stage_bytes;
         pull_frame(sb, tx + 1, ty + 1, X);
-        ring[q & 3][0][ty + 1][tx + 1] = node_density<L, C>(X[0]);
-        ring[q & 3][1][ty + 1][tx + 1] = node_density<L, C>(X[1]);
+        ring[q & 3][ty + 1][tx + 1] = node_densities<L, C>(X);
         if (halo) {
             if constexpr (kSplit) {
-                ring[q & 3][hs][hfy][hfx] = tma_density<TX, TY, S, St>(sb, hs, hfx, hfy, hs == 0 ? a.ref_A : a.ref_B);
+                (&ring[q & 3][hfy][hfx].a)[hs] = tma_density<TX, TY, S, St>(sb, hs, hfx, hfy, hs == 0 ? a.ref_A : a.ref_B);
             } else {
                 C h[2][Q];
                 pull_frame(sb, hfx, hfy, h);
-                ring[q & 3][0][hfy][hfx] = node_density<L, C>(h[0]);
-                ring[q & 3][1][hfy][hfx] = node_density<L, C>(h[1]);
+                ring[q & 3][hfy][hfx] = node_densities<L, C>(h);
             }
         }
     };
     auto collide = [&](int q, C (&X)[2][Q]) {
         // ring slots of the planes z - 1, z, z + 1 (steps q - 1 and q + 1 swap roles downwards)
         const int sc = q & 3, sm_ = (down ? q + 1 : q - 1) & 3, sp = (down ? q - 1 : q + 1) & 3;
-        const C rA = ring[sc][0][ty + 1][tx + 1];
-        const C rB = ring[sc][1][ty + 1][tx + 1];
-        auto nbr = [&](int s, int i) -> C {
+        const Two<C> r = ring[sc][ty + 1][tx + 1];
+        const C rA = r.a, rB = r.b;
+        auto nbr = [&](int i) -> Two<C> {
             const int sl = L::c(i, 2) == 0 ? sc : (L::c(i, 2) > 0 ? sp : sm_);
-            return ring[sl][s][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
+            return ring[sl][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
         };
         if constexpr (FORCING == kSchemeFE) {
             C gp[3], lp;
@@ -390,7 +388,7 @@ __device__ __forceinline__ int tma_item(const CUtensorMap* pmap, const CUtensorM
             if constexpr (FORCING == kForcingGuo)
                 node_collide_guo<L, C>(X, rA, rB, gA, gB, a.omega_A, a.omega_B);
             else
-                node_collide<L, C>(X, rA, rB, gA, gB, a.omega_A, a.omega_B, a.tau_A, a.tau_B);
+                node_collide<L, C, std::is_same<St, float>::value>(X, rA, rB, gA, gB, a.omega_A, a.omega_B, a.tau_A, a.tau_B);
         }
         if (owner) store_node<L, St>(a, gx, gy, zof(q), X, rA, rB);
     };
