@@ -62,9 +62,8 @@ cudaError_t launch_batch(const void* lats, const BatchItem* items, int nitems, i
     long long grid = grid_mode ? nitems : (long long)sm_count * per_sm;
     if (grid > nitems) grid = nitems;
     if (grid < 1) return cudaSuccess;
-    kern<<<(unsigned)grid, dim3(TX, TY), 0, st>>>(static_cast<const BatchLattice<S>*>(lats), items, nitems, parity,
-                                                  grid_mode ? nullptr : ctr);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)grid), dim3(TX, TY), 0, st, 1, 1,
+                          static_cast<const BatchLattice<S>*>(lats), items, nitems, parity, grid_mode ? nullptr : ctr);
 }
 
 template <int TX, int TY, int ST>
@@ -78,9 +77,8 @@ cudaError_t launch_batch_tma(const void* lats, const BatchItem* items, int nitem
     long long grid = grid_mode ? nitems : sm_count;
     if (grid > nitems) grid = nitems;
     if (grid < 1) return cudaSuccess;
-    kern<<<(unsigned)grid, dim3(TX, TY), T::smem_bytes, st>>>(static_cast<const BatchTmaLattice*>(lats), items,
-                                                              nitems, parity, grid_mode ? nullptr : ctr);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)grid), dim3(TX, TY), T::smem_bytes, st, 1, 1,
+                          static_cast<const BatchTmaLattice*>(lats), items, nitems, parity, grid_mode ? nullptr : ctr);
 }
 
 template <int WX, int WY, int NX, int NY, int S>
@@ -93,8 +91,8 @@ cudaError_t launch_batch_tma_mixed(const void* lats, const BatchItem* items, int
     const cudaError_t attr = dynamic_smem_once<kern>((int)smem);
     if (attr != cudaSuccess) return attr;
     if (nitems < 1) return cudaSuccess;
-    kern<<<(unsigned)nitems, WX * WY, smem, st>>>(static_cast<const BatchTmaLattice*>(lats), items, nitems, parity);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)nitems), dim3(WX * WY), smem, st, 1, 1,
+                          static_cast<const BatchTmaLattice*>(lats), items, nitems, parity);
 }
 
 template <int S>
@@ -106,8 +104,8 @@ cudaError_t launch_batch_tma_shape3(const void* lats, const BatchItem* items, in
     const cudaError_t attr = dynamic_smem_once<kern>((int)smem);
     if (attr != cudaSuccess) return attr;
     if (nitems < 1) return cudaSuccess;
-    kern<<<(unsigned)nitems, 384, smem, st>>>(static_cast<const BatchTmaLattice*>(lats), items, nitems, parity);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)nitems), dim3(384), smem, st, 1, 1,
+                          static_cast<const BatchTmaLattice*>(lats), items, nitems, parity);
 }
 
 template <class St>
@@ -117,9 +115,8 @@ cudaError_t launch_batch_tma_rest(const void* lats, const BatchItem* items, int 
     const cudaError_t attr = dynamic_smem_once<kern>((int)T::smem_bytes);
     if (attr != cudaSuccess) return attr;
     if (nitems < 1) return cudaSuccess;
-    kern<<<(unsigned)nitems, 256, T::smem_bytes, st>>>(static_cast<const BatchTmaRestLattice<St>*>(lats), items,
-                                                        nitems, parity);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)nitems), dim3(256), T::smem_bytes, st, 1, 1,
+                          static_cast<const BatchTmaRestLattice<St>*>(lats), items, nitems, parity);
 }
 
 template <class L, class S>

@@ -68,6 +68,8 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     const bool halo = tid < H;
     int hfx, hfy;
     halo_cell<TX, TY>(tid, hfx, hfy);
+    chain_wait();
+    chain_next();
     BatchQueue queue{ctr, &s_next, 0};
     queue.fetch(tid);
     __syncthreads();
@@ -165,6 +167,8 @@ __global__ void __launch_bounds__(TX* TY, 1)
     __shared__ int s_next;
     TmaSmem<TX, TY, S> sm(smem_raw);
     const int tid = threadIdx.y * TX + threadIdx.x;
+    chain_wait();
+    chain_next();
     BatchQueue queue{ctr, &s_next, 0};
     queue.fetch(tid);  // the first item
     sm.init_barriers();  // (ends with a CTA barrier)
@@ -245,11 +249,15 @@ __global__ void __launch_bounds__(WX* WY, 1)
     if (l->wide) {
         TmaSmem<WX, WY, S> sm(smem_raw);
         sm.init_barriers();
+        chain_wait();
+        chain_next();
         tma_item<WX, WY, S>(&l->map[parity], nullptr, a, w.x0, w.y0, w.z0, 0u, sm, l->err, false, nullptr,
                             TmaNoHook(), true);
     } else {
         TmaSmem<NX, NY, S> sm(smem_raw);
         sm.init_barriers();
+        chain_wait();
+        chain_next();
         tma_item<NX, NY, S>(&l->map[parity], nullptr, a, w.x0, w.y0, w.z0, 0u, sm, l->err, false, nullptr,
                             TmaNoHook(), true);
     }
@@ -275,16 +283,22 @@ __global__ void __launch_bounds__(384, 1)
     if (l->wide == 1) {
         TmaSmem<64, 6, S> sm(smem_raw);
         sm.init_barriers();
+        chain_wait();
+        chain_next();
         tma_item<64, 6, S>(&l->map[parity], nullptr, a, w.x0, w.y0, w.z0, 0u, sm, l->err, false, nullptr,
                            TmaNoHook(), true);
     } else if (l->wide == 2) {
         TmaSmem<48, 8, S> sm(smem_raw);
         sm.init_barriers();
+        chain_wait();
+        chain_next();
         tma_item<48, 8, S>(&l->map[parity], nullptr, a, w.x0, w.y0, w.z0, 0u, sm, l->err, false, nullptr,
                            TmaNoHook(), true);
     } else {
         TmaSmem<32, 12, S> sm(smem_raw);
         sm.init_barriers();
+        chain_wait();
+        chain_next();
         tma_item<32, 12, S>(&l->map[parity], nullptr, a, w.x0, w.y0, w.z0, 0u, sm, l->err, false, nullptr,
                             TmaNoHook(), true);
     }
@@ -317,6 +331,8 @@ __global__ void __launch_bounds__(256, 2)
     }
     TmaSmem<32, 8, 2, St> sm(smem_raw);
     sm.init_barriers();
+    chain_wait();
+    chain_next();
     tma_item<32, 8, 2, St>(&l->maps[parity].pop, &l->maps[parity].rho, a, w.x0, w.y0, w.z0, 0u, sm, l->err, false,
                            nullptr, TmaNoHook(), true);
 }

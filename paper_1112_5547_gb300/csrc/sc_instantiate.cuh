@@ -21,16 +21,14 @@ cudaError_t step_tiled(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) 
     // 0.67 ms a step at 4096^2; two (128 registers) in FP64.
     constexpr int kMin = L::D == 2 ? (sizeof(C) == 8 ? 2 : 3) * (TX * TY <= 128 ? 2 : 1) / (TX * TY > 256 ? 2 : 1)
                          : sizeof(C) == 8 ? 1 : (TX * TY <= 128 ? 4 : (TX * TY <= 256 ? 2 : 1));
-    sc_fused_kernel<L, S, TX, TY, kModeStep, kMin><<<step_grid(p), dim3(TX, TY), 0, st>>>(a, fo);
-    return cudaGetLastError();
+    return launch_chained(sc_fused_kernel<L, S, TX, TY, kModeStep, kMin>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a, fo);
 }
 
 template <class L, class S, int TX, int TY, int MINB>
 cudaError_t step_reload(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) {
     using C = typename Codec<S>::C;
     constexpr int kMin = sizeof(C) == 8 ? (MINB > 2 ? MINB / 2 : 1) : MINB;
-    sc_step_reload_kernel<L, S, TX, TY, kMin><<<step_grid(p), dim3(TX, TY), 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(sc_step_reload_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a);
 }
 
 template <class L, class S, int TX, int TY, int ST, int FORCING = kForcingShift, int MINB = 1> struct TmaLaunch {
@@ -54,23 +52,7 @@ template <class S, int TX, int TY, int ST, int FORCING, int MINB> struct TmaLaun
             auto kern = sc_step_tma_kernel<TX, TY, ST, S, FORCING, MINB>;
             e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
             if (e != cudaSuccess) return e;
-            if (ts.cx == 1 && ts.cy == 1) {
-                kern<<<step_grid(p), dim3(TX, TY), T::smem_bytes, st>>>(maps, a, p.err);
-                return cudaGetLastError();
-            }
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = step_grid(p);
-            cfg.blockDim = dim3(TX, TY);
-            cfg.dynamicSmemBytes = T::smem_bytes;
-            cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = ts.cx;
-            attr[0].val.clusterDim.y = ts.cy;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            return cudaLaunchKernelEx(&cfg, kern, maps, a, p.err);
+            return launch_chained(kern, step_grid(p), dim3(TX, TY), T::smem_bytes, st, ts.cx, ts.cy, maps, a, p.err);
         }
     }
 };
@@ -83,8 +65,7 @@ template <class S, int TX, int TY, int MINB> struct RegPipeLaunch<D3Q19, S, TX, 
         if constexpr (sizeof(S) == 8) {
             return cudaErrorInvalidValue;  // three planes of doubles do not fit in registers
         } else {
-            sc_step_regpipe_kernel<S, TX, TY, MINB><<<step_grid(p), dim3(TX, TY), 0, st>>>(a);
-            return cudaGetLastError();
+            return launch_chained(sc_step_regpipe_kernel<S, TX, TY, MINB>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a);
         }
     }
 };

@@ -45,8 +45,8 @@ __device__ __forceinline__ void pull_node(const LatticeArgs<S>& a, int x, int y,
         // x - c_x and y - c_y lie in [-1, n]: the ghost images make them valid
         const size_t node = cell(a, x - L::c(i, 0), y - L::c(i, 1), zs[L::c(i, 2) + 1]);
         if constexpr (Codec<S>::kRest) {
-            const uint32_t v = __ldg(&(a.fin + (size_t)i * (size_t)a.Np + node)->v);
-            rest_decode<S>(v, (C)L::w(i), __ldg(rest_rho<L>(a.fin, a.Np) + node), f[0][i], f[1][i]);
+            const uint32_t v = (a.fin + (size_t)i * (size_t)a.Np + node)->v;
+            rest_decode<S>(v, (C)L::w(i), rest_rho<L>(a.fin, a.Np)[node], f[0][i], f[1][i]);
         } else {
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
@@ -170,6 +170,10 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     constexpr int H = 2 * FX + 2 * TY;
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
     __shared__ Two<C> srho[NPL][FY][FX];  // densities (rho_A, rho_B)
+    if (MODE == kModeStep) {
+        chain_wait();
+        chain_next();
+    }
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -354,6 +358,8 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
     constexpr int H = 2 * FX + 2 * TY;
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
     __shared__ Two<C> ring[NPL][FY][FX];
+    chain_wait();
+    chain_next();
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;

@@ -58,6 +58,8 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_regpipe_kernel(const Lat
 
     __shared__ __align__(16) W hst[Q2][H];
     __shared__ Two<C> ring[4][FY][FX];
+    chain_wait();
+    chain_next();
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;

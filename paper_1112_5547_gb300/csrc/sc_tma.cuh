@@ -360,7 +360,7 @@ __device__ __forceinline__ int tma_item(const CUtensorMap* pmap, const CUtensorM
         ring[q & 3][ty + 1][tx + 1] = node_densities<L, C>(X);
         if (halo) {
             if constexpr (kSplit) {
-                (&ring[q & 3][hfy][hfx].a)[hs] = tma_density<TX, TY, S, St>(sb, hs, hfx, hfy, hs == 0 ? a.ref_A : a.ref_B);
+                reinterpret_cast<float*>(&ring[q & 3][hfy][hfx])[hs] = tma_density<TX, TY, S, St>(sb, hs, hfx, hfy, hs == 0 ? a.ref_A : a.ref_B);
             } else {
                 C h[2][Q];
                 pull_frame(sb, hfx, hfy, h);
@@ -470,6 +470,8 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     extern __shared__ unsigned char smem_raw[];
     TmaSmem<TX, TY, S, St> sm(smem_raw);
     sm.init_barriers();
+    chain_wait();
+    chain_next();
     tma_item<TX, TY, S, St, TmaNoHook, FORCING>(&maps.pop, &maps.rho, a, blockIdx.x * TX, blockIdx.y * TY,
                                                 blockIdx.z * a.zchunk, 0u, sm, err);
 }
