@@ -12,6 +12,7 @@
 
 #include "../../include/lbm_sc.h"
 #include "sc_launch.cuh"
+#include "sc_shape.h"
 
 using lbmsc::Plan;
 
@@ -86,7 +87,7 @@ int pick_zchunk(const lbm_sc_params* p, int tx = lbmsc::kTX, int ty = lbmsc::kTY
 }
 
 Plan make_plan(const lbm_sc_params* p) {
-    Plan pl;
+    Plan pl{};
     pl.lattice = p->lattice;
     pl.precision = p->precision;
     pl.nx = p->nx;
@@ -94,8 +95,6 @@ Plan make_plan(const lbm_sc_params* p) {
     pl.nz = p->nz;
     pl.N = (long long)p->nx * p->ny * p->nz;
     pl.zchunk = pick_zchunk(p);
-    pl.step_tile = 0;
-    pl.step_zchunk = pl.zchunk;
     pl.sm_count = 152;
     pl.tau_A = p->tau_A;
     pl.tau_B = p->tau_B;
@@ -110,6 +109,7 @@ Plan make_plan(const lbm_sc_params* p) {
     pl.gamma = p->gamma;
     lbmsc::storage_geometry(p->nx, p->ny, p->nz, (int)store_bytes(p->precision), pl.px, pl.py, pl.gxo, pl.gyo,
                             pl.Np);
+    lbmsc::pick_step(pl);
     return pl;
 }
 
@@ -184,10 +184,14 @@ lbm_status lbm_sc_create(const lbm_sc_params* p, void* d_workspace, size_t works
         // the default when no device is present (host-only use)
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
-            h->plan.sm_count = sms;
-        else
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
+            if (sms != h->plan.sm_count) {
+                h->plan.sm_count = sms;
+                lbmsc::pick_step(h->plan);
+            }
+        } else {
             cudaGetLastError();
+        }
     }
     *out = h;
     return LBM_OK;
