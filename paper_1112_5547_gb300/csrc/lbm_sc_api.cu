@@ -18,6 +18,8 @@ using lbmsc::Plan;
 
 // Slabs of z planes lbm_sc_run_host overlaps its host copies with (at most).
 constexpr int kIoSlabs = 8;
+// Steps of one launch of the resident D2Q9 kernel (at most; some milliseconds).
+constexpr int kStepsPerLaunch = 4096;
 
 struct lbm_sc_handle {
     lbm_sc_params params;
@@ -246,7 +248,31 @@ lbm_status lbm_sc_init_fields(lbm_sc_handle* h, const void* d_rhoA, const void* 
 
 lbm_status lbm_sc_step(lbm_sc_handle* h, int nsteps) {
     if (!h || nsteps < 0) return LBM_ERR_INVALID_ARG;
-    for (int t = 0; t < nsteps; ++t) {
+    int left = nsteps;
+    // D2Q9 FP32 on its default tile: all steps in one launch, or two per launch.
+    // Buffers change places with every odd number of steps as in single steps
+    // (pairs are taken two at a time), so callers that count steps find the
+    // populations where they were.
+    if (h->plan.lattice == LBM_D2Q9 && h->plan.precision == LBM_F32 && h->plan.step_tile == lbmsc::kTileD2) {
+        if (left >= 3 && lbmsc::d2q9_resident_fits(h->plan)) {
+            while (left > 0) {
+                const int n = left < kStepsPerLaunch ? left : kStepsPerLaunch;
+                const int to = h->cur ^ (n & 1);
+                if (lbmsc::d2q9_resident(h->plan, h->buf[h->cur], h->buf[to], n, h->stream) != cudaSuccess)
+                    return LBM_ERR_CUDA;
+                h->cur = to;
+                left -= n;
+            }
+        } else if (lbmsc::d2_pair_fits(h->plan)) {
+            for (; left >= 4; left -= 4)
+                for (int k = 0; k < 2; ++k) {
+                    if (lbmsc::d2q9_pair(h->plan, h->buf[h->cur], h->buf[1 - h->cur], h->stream) != cudaSuccess)
+                        return LBM_ERR_CUDA;
+                    h->cur = 1 - h->cur;
+                }
+        }
+    }
+    for (; left > 0; --left) {
         const cudaError_t e = launch_step(h->plan, h->buf[h->cur], h->buf[1 - h->cur], h->stream);
         if (e != cudaSuccess) return LBM_ERR_CUDA;
         h->cur = 1 - h->cur;
@@ -612,6 +638,7 @@ struct lbm_sc_batch {
     int* d_ctr;  // work-queue counters of the batch kernels
     int nitems;
     int parity;
+    bool pairs;  // two steps per launch where they come in fours (batch_pair)
     int sm_count;
     cudaStream_t stream;
     cudaGraphExec_t graph[2];  // graph_steps launches starting at parity 0 / 1
@@ -663,7 +690,15 @@ std::vector<lbmsc::BatchItem> batch_items(lbm_sc_handle* const* handles, int n, 
 }
 
 cudaError_t batch_launch_steps(lbm_sc_batch* b, int nsteps) {
-    for (int t = 0; t < nsteps; ++t) {
+    int left = nsteps;
+    if (b->pairs)  // two pairs at a time: the parity counts steps
+        for (; left >= 4; left -= 4)
+            for (int k = 0; k < 2; ++k) {
+                const cudaError_t e = lbmsc::batch_pair(b->d_lats, b->d_items, b->nitems, b->parity, b->stream);
+                if (e != cudaSuccess) return e;
+                b->parity ^= 1;
+            }
+    for (; left > 0; --left) {
         const cudaError_t e = lbmsc::batch_step(b->lattice, b->precision, b->tile, b->d_lats, b->d_items, b->nitems,
                                                 b->parity, b->sm_count, b->d_ctr, b->stream);
         if (e != cudaSuccess) return e;
@@ -700,6 +735,8 @@ lbm_status lbm_sc_batch_create(lbm_sc_handle* const* handles, int n, int tile, i
     b->zchunk = zchunk;
     b->graph_steps = graph_steps;
     b->parity = 0;
+    b->pairs = true;
+    for (int k = 0; k < n; ++k) b->pairs = b->pairs && lbmsc::batch_pair_fits(tile, handles[k]->plan);
     b->sm_count = handles[0]->plan.sm_count;
     b->stream = static_cast<cudaStream_t>(cuda_stream);
     b->graph[0] = b->graph[1] = nullptr;
@@ -729,6 +766,7 @@ lbm_status lbm_sc_batch_create(lbm_sc_handle* const* handles, int n, int tile, i
     if (e == cudaSuccess)
         e = lbmsc::batch_step(b->lattice, b->precision, tile, b->d_lats, b->d_items, 0, 0, b->sm_count, b->d_ctr,
                               b->stream);
+    if (e == cudaSuccess && b->pairs) e = lbmsc::batch_pair(b->d_lats, b->d_items, 0, 0, b->stream);
     if (e != cudaSuccess) {
         delete b;
         return LBM_ERR_CUDA;

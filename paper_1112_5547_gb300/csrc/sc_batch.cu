@@ -4,6 +4,7 @@
 #include <type_traits>
 
 #include "sc_batch.cuh"
+#include "sc_d2.cuh"
 #include "sc_batch_launch.h"
 #include "sc_args.cuh"
 
@@ -254,6 +255,13 @@ cudaError_t batch_lattice_fill(const Plan& p, const void* b0, const void* b1, in
         default: return cudaErrorInvalidValue;
     }
     return cudaSuccess;
+}
+
+cudaError_t batch_pair(const void* lats, const BatchItem* items, int nitems, int parity, cudaStream_t st) {
+    const cudaError_t attr = dynamic_smem_once<sc_d2_pair_batch_kernel<kPairThreads>>((int)sizeof(PairSmem));
+    if (attr != cudaSuccess || nitems < 1) return attr;
+    return launch_chained(sc_d2_pair_batch_kernel<kPairThreads>, dim3((unsigned)nitems), dim3(kPairThreads), sizeof(PairSmem), st, 1, 1,
+                          static_cast<const BatchLattice<float>*>(lats), items, parity);
 }
 
 cudaError_t batch_step(int lattice, int precision, int tile, const void* lats, const BatchItem* items, int nitems,

@@ -94,6 +94,10 @@ inline bool batch_tile_fits(int tile, const Plan& p) {
 size_t batch_lattice_bytes(int precision, int tile);
 cudaError_t batch_lattice_fill(const Plan& p, const void* b0, const void* b1, int cur0, int zchunk, int tile,
                                void* dst);
+// Whether a batch of these tiles can take two steps per launch (sc_d2.cuh), and
+// the launch: FP32 D2Q9 with 32-wide tiles, every lattice of a two-step frame.
+inline bool batch_pair_fits(int tile, const Plan& p) { return (tile == 0 || tile == 1 || tile == 7) && d2_pair_fits(p); }
+cudaError_t batch_pair(const void* lats, const BatchItem* items, int nitems, int parity, cudaStream_t st);
 // ctr: two device ints, zero before the first launch (each launch leaves them zero).
 cudaError_t batch_step(int lattice, int precision, int tile, const void* lats, const BatchItem* items, int nitems,
                        int parity, int sm_count, int* ctr, cudaStream_t st);

@@ -198,6 +198,19 @@ inline long long fused_blocks(const Plan& p) {
 }
 
 cudaError_t d2q9_step(const Plan& p, const void* fin, void* fout, cudaStream_t st);
+// The tile of an untuned D2Q9 lattice in 32- and 16-bit storage.
+constexpr int kTileD2 = 3;
+// Several D2Q9 FP32 steps per launch (sc_d2.cuh).  Two steps: lattices at least
+// as wide and high as the tile's frame.  nsteps steps (fout may be fin): lattices
+// that fit a cluster's shared memory and are small enough to be better off on
+// its 16 SMs.
+constexpr int kPairTX = 32, kPairTY = 16, kPairThreads = 384;
+inline bool d2_pair_fits(const Plan& p) {
+    return p.lattice == 0 && p.precision == 1 && p.nx >= kPairTX + 6 && p.ny >= kPairTY + 6;
+}
+cudaError_t d2q9_pair(const Plan& p, const void* fin, void* fout, cudaStream_t st);
+bool d2q9_resident_fits(const Plan& p);
+cudaError_t d2q9_resident(const Plan& p, const void* fin, void* fout, int nsteps, cudaStream_t st);
 // init of planes [zlo, zhi) (zhi = 0: all planes)
 cudaError_t d2q9_init(const Plan& p, const void* rA, const void* rB, const void* u, void* fout,
                       cudaStream_t st, int zlo = 0, int zhi = 0);

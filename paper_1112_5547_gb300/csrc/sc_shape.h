@@ -141,7 +141,7 @@ inline void pick_step(Plan& p) {
         // D2Q9: 32x4 tiles, four to six CTAs per SM (4096^2 FP32 0.461 ms a
         // step against 0.487 with 32x8, 64^2 2.7 us against 3.2); FP64 is
         // bound by its units and 32x8 has the smaller halo (256^2 30.5 / 31.2 us)
-        p.step_tile = p.precision == 0 ? 0 : 3;
+        p.step_tile = p.precision == 0 ? 0 : kTileD2;
         p.step_zchunk = 1;
         return;
     }

@@ -75,3 +75,44 @@ def test_untuned_equals_one_register_kernel(lat, sizes, prec):
                 for u, v in zip(x, y):
                     assert np.isfinite(v).all()
                     np.testing.assert_array_equal(u, v)
+
+
+@pytest.mark.gpu
+def test_many_steps_per_launch_equal_single_steps():
+    """D2Q9 FP32: all steps in one cluster, two steps per launch, and both in a batch,
+    for every remainder of the steps, against single steps of another tile."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1112_5547_gb300 import build, inputs, lbm_sc as lib
+    build.build()
+    G = 2.4 / 1.04
+    # cluster kernel: one row band per CTA at least two rows high, ragged bands, wide and narrow rows, many steps
+    # two-step tile: smallest frame, one more and one less than whole tiles
+    shapes = [(4, 3), (5, 40), (33, 64), (8, 512), (100, 100), (22, 38), (22, 600), (161, 129), (192, 160), (127, 161)]
+    for shape in shapes:
+        for kw in ({}, {"forcing": "guo", "body_A": 1e-4}):
+            f = inputs.drop(shape, min(shape) / 3.0, seed=6, dtype=np.float32)
+            a = _run(lib, 0, shape, "f32", kw, None, f, (2, 3, 4, 5, 11))
+            b = _run(lib, 0, shape, "f32", kw, (0, 1), f, (2, 3, 4, 5, 11))
+            for x, y in zip(a, b):
+                for u, v in zip(x, y):
+                    np.testing.assert_array_equal(u, v)
+    f = inputs.drop((8, 32), 2.0, seed=7, dtype=np.float32)  # more steps than one launch takes
+    for u, v in zip(_run(lib, 0, (8, 32), "f32", {}, None, f, (4101,))[0],
+                    _run(lib, 0, (8, 32), "f32", {}, (0, 1), f, (4101,))[0]):
+        np.testing.assert_array_equal(u, v)
+    stream = torch.cuda.Stream()
+    shapes = [(64, 64), (22, 38), (100, 40), (257, 130)]
+    fields = [inputs.drop(s, min(s) / 3.0, seed=8 + k, dtype=np.float32) for k, s in enumerate(shapes)]
+    for tile, graph in ((0, 0), (1, 8), (7, 8)):
+        for n in (4, 7, 18):
+            with torch.cuda.stream(stream):
+                solo = [lib.Lattice(0, s, 1.0, 0.9, G, "f32", stream=stream).set_tuning(0).init(*f).step(n)
+                        for s, f in zip(shapes, fields)]
+                lats = [lib.Lattice(0, s, 1.0, 0.9, G, "f32", stream=stream).init(*f) for s, f in zip(shapes, fields)]
+                b = lib.Batch(lats, tile=tile, graph_steps=graph, stream=stream).step(n)
+                for u, v in zip(solo, lats):
+                    for x, y in zip(u.moments(), v.moments()):
+                        assert torch.equal(x, y)
+                b.close()
