@@ -96,7 +96,6 @@ Plan make_plan(const lbm_sc_params* p) {
     pl.ny = p->ny;
     pl.nz = p->nz;
     pl.N = (long long)p->nx * p->ny * p->nz;
-    pl.zchunk = pick_zchunk(p);
     pl.sm_count = 152;
     pl.tau_A = p->tau_A;
     pl.tau_B = p->tau_B;
@@ -126,7 +125,7 @@ size_t population_bytes(const lbm_sc_params* p) {
 }
 
 size_t partial_bytes(const Plan& pl) {
-    return (size_t)lbmsc::fused_blocks(pl) * lbmsc::kNumDiag * sizeof(double);
+    return (size_t)lbmsc::diag_parts(pl) * lbmsc::kNumDiag * sizeof(double);
 }
 
 lbm_status cuda_status(cudaError_t e) { return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA; }
@@ -313,7 +312,7 @@ lbm_status lbm_sc_diagnostics(lbm_sc_handle* h, const lbm_sc_window* window, lbm
     }
     cudaError_t e = launch_moments(h->plan, h->buf[h->cur], o, h->stream);
     if (e != cudaSuccess) return LBM_ERR_CUDA;
-    e = lbmsc::diag_finish(h->partials, lbmsc::fused_blocks(h->plan), h->result, h->stream);
+    e = lbmsc::diag_finish(h->partials, lbmsc::diag_parts(h->plan), h->result, h->stream);
     if (e != cudaSuccess) return LBM_ERR_CUDA;
     double r[lbmsc::kNumDiag];
     int err_word = 0;
@@ -521,13 +520,11 @@ lbm_status lbm_sc_run_host(lbm_sc_handle* h, void* d_staging, size_t staging_byt
     const cudaStream_t ms = h->stream, cs = h->io_stream;
     auto ok = [](cudaError_t e) { return e == cudaSuccess; };
     // z slabs: the host copies of one slab overlap the kernels of another.
-    // Moments slabs are whole chunks of 32 planes (their own z chunking).
-    Plan mp = h->plan;
-    if (nz >= 64) mp.zchunk = 32;
-    const int chunks = (nz + mp.zchunk - 1) / mp.zchunk;
+    // Slabs are whole multiples of 32 planes.
+    const int slab = nz >= 64 ? 32 : nz, chunks = (nz + slab - 1) / slab;
     const int nslab = nz >= 64 ? (chunks < kIoSlabs ? chunks : kIoSlabs) : 1;  // no empty slab
     int zb[kIoSlabs + 1];
-    for (int k = 0; k <= nslab; ++k) zb[k] = (int)((long long)chunks * k / nslab) * mp.zchunk;
+    for (int k = 0; k <= nslab; ++k) zb[k] = (int)((long long)chunks * k / nslab) * slab;
     zb[nslab] = nz;
     auto copy_planes = [&](char* dev, const void* host, int z0, int z1, int nfield, cudaMemcpyKind kind) {
         // planes [z0, z1) of nfield consecutive fields of fb bytes each
@@ -578,7 +575,7 @@ lbm_status lbm_sc_run_host(lbm_sc_handle* h, void* d_staging, size_t staging_byt
         o.win[4] = 1e300;
         o.zlo = zb[k];
         o.zhi = zb[k + 1];
-        if (launch_moments(mp, h->buf[h->cur], o, ms) != cudaSuccess) return LBM_ERR_CUDA;
+        if (launch_moments(h->plan, h->buf[h->cur], o, ms) != cudaSuccess) return LBM_ERR_CUDA;
         if (!ok(cudaEventRecord(h->io_out[k], ms)) || !ok(cudaStreamWaitEvent(cs, h->io_out[k], 0))) return LBM_ERR_CUDA;
         if ((h_rhoA_out && !copy_planes(dA, h_rhoA_out, zb[k], zb[k + 1], 1, d2h)) ||
             (h_rhoB_out && !copy_planes(dB, h_rhoB_out, zb[k], zb[k + 1], 1, d2h)) ||

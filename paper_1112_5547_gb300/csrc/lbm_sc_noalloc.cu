@@ -12,8 +12,8 @@
 
 namespace {
 
-// Largest diagnostics grid the static scratch holds: one slot of kNumDiag
-// doubles per CTA of the moments kernel (2.1 MiB in total on every device that
+// Records the static scratch holds: kNumDiag doubles per CTA of the moments
+// kernel (2.1 MiB in total on every device that
 // loads the library, held until the process exits).
 constexpr long long kStaticDiagSlots = 16384;
 
@@ -56,9 +56,8 @@ extern "C" LBM_SC_API lbm_status lbm_sc_diagnostics_noalloc(const lbm_sc_params*
     pl.ny = p->ny;
     pl.nz = p->nz;
     pl.N = (long long)p->nx * p->ny * p->nz;
-    pl.zchunk = p->lattice == LBM_D3Q19 ? p->nz : 1;  // one CTA per tile column: fewest partials
     pl.step_tile = 0;
-    pl.step_zchunk = pl.zchunk;
+    pl.step_zchunk = 1;
     pl.sm_count = 152;
     pl.tau_A = p->tau_A;
     pl.tau_B = p->tau_B;
@@ -73,8 +72,13 @@ extern "C" LBM_SC_API lbm_status lbm_sc_diagnostics_noalloc(const lbm_sc_params*
     lbmsc::storage_geometry(p->nx, p->ny, p->nz, lbmsc::storage_elem_bytes(p->precision), pl.px, pl.py, pl.gxo, pl.gyo, pl.Np);
     pl.err = nullptr;
 
-    const long long parts = lbmsc::fused_blocks(pl);
-    if (parts > kStaticDiagSlots) return LBM_ERR_INVALID_ARG;  // larger than the static scratch
+    // one slot per tile column is what the scratch was made for: more are refused
+    // (the launch itself leaves at most kDiagCtas records)
+    const long long columns =
+        (long long)((p->nx + lbmsc::kTX - 1) / lbmsc::kTX) * ((p->ny + lbmsc::kTY - 1) / lbmsc::kTY);
+    if (columns > kStaticDiagSlots) return LBM_ERR_INVALID_ARG;
+    const long long parts = lbmsc::diag_parts(pl);
+    static_assert(lbmsc::kDiagCtas <= kStaticDiagSlots, "diagnostics records fit the static scratch");
 
     double* scratch = nullptr;
     if (device_scratch(&scratch) != cudaSuccess) return LBM_ERR_CUDA;

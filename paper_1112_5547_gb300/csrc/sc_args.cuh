@@ -16,7 +16,7 @@ template <class S> LatticeArgs<S> make_args(const Plan& p, const void* fin, void
     a.nx = p.nx;
     a.ny = p.ny;
     a.nz = p.nz;
-    a.zchunk = p.zchunk;
+    a.zchunk = p.step_zchunk;
     a.zbase = 0;
     a.zend = p.nz;
     a.N = p.N;

@@ -77,7 +77,7 @@ cudaError_t d2q9_moments(const Plan& p, const void* fin, const MomentsOut& o, cu
     return moments_any<D2Q9>(p, fin, o, st);
 }
 cudaError_t diag_finish(const double* partials, long long nparts, double* out, cudaStream_t st) {
-    sc_diag_finish_kernel<256><<<1, 256, 0, st>>>(partials, nparts, out);
+    sc_diag_finish_kernel<256><<<kNumDiag, 256, 0, st>>>(partials, nparts, out);
     return cudaGetLastError();
 }
 }  // namespace lbmsc

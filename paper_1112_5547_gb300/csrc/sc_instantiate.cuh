@@ -14,14 +14,13 @@ namespace lbmsc {
 template <class L, class S, int TX, int TY>
 cudaError_t step_tiled(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) {
     using C = typename Codec<S>::C;
-    FieldArgs<C> fo{};
     // register budget: 65536 / (threads * CTAs per SM).  A D2Q9 CTA holds one
     // row block and no pipeline, so its loads in flight are its warps': three
     // CTAs of 256 threads (80 registers) rather than two (90), 0.50 against
     // 0.67 ms a step at 4096^2; two (128 registers) in FP64.
     constexpr int kMin = L::D == 2 ? (sizeof(C) == 8 ? 2 : 3) * (TX * TY <= 128 ? 2 : 1) / (TX * TY > 256 ? 2 : 1)
                          : sizeof(C) == 8 ? 1 : (TX * TY <= 128 ? 4 : (TX * TY <= 256 ? 2 : 1));
-    return launch_chained(sc_fused_kernel<L, S, TX, TY, kModeStep, kMin>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a, fo);
+    return launch_chained(sc_fused_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a);
 }
 
 template <class L, class S, int TX, int TY, int MINB>
@@ -175,11 +174,10 @@ cudaError_t init_typed(const Plan& p, const void* rA, const void* rB, const void
     const LatticeArgs<S> a = make_args<S>(p, nullptr, fout);
     if (zhi <= 0 || zhi > p.nz) zhi = p.nz;
     if (zlo < 0 || zlo >= zhi) return zlo == zhi ? cudaSuccess : cudaErrorInvalidValue;
-    long long blocks = ((long long)p.nx * p.ny * (zhi - zlo) + 255) / 256;
-    if (blocks > 152 * 64) blocks = 152 * 64;
-    if (blocks < 1) blocks = 1;
-    sc_init_kernel<L, S><<<(unsigned)blocks, 256, 0, st>>>(a, static_cast<const C*>(rA), static_cast<const C*>(rB),
-                                                          static_cast<const C*>(u), zlo, zhi);
+    const long long rows = (long long)(p.ny + 4) * (zhi - zlo);
+    const dim3 grid((unsigned)((p.nx + 2 * kInitLead + kInitThreads - 1) / kInitThreads), (unsigned)(rows < 32768 ? rows : 32768));
+    sc_init_kernel<L, S><<<grid, kInitThreads, 0, st>>>(a, static_cast<const C*>(rA), static_cast<const C*>(rB),
+                                                        static_cast<const C*>(u), zlo, zhi);
     return cudaGetLastError();
 }
 
@@ -198,15 +196,21 @@ cudaError_t moments_typed(const Plan& p, const void* fin, const MomentsOut& o, c
     fo.win_c[2] = o.win[2];
     fo.r_in2 = o.win[3] < 0 ? -1.0 : o.win[3] * o.win[3];
     fo.r_out2 = o.win[4] * o.win[4];
-    dim3 grid = fused_grid(p);
     if (o.zhi > 0) {
-        // planes [zlo, zhi) only (whole chunks of p.zchunk from zlo; fields only, no partials)
+        // planes [zlo, zhi) only (fields only, no partials)
         if (o.partials || o.zlo < 0 || o.zlo >= o.zhi || o.zhi > p.nz) return cudaErrorInvalidValue;
         a.zbase = o.zlo;
         a.zend = o.zhi;
-        grid.z = (unsigned)((o.zhi - o.zlo + p.zchunk - 1) / p.zchunk);
     }
-    sc_fused_kernel<L, S, kTX, kTY, kModeMoments, 1><<<grid, dim3(kTX, kTY), 0, st>>>(a, fo);
+    const MomentsShape m = moments_shape(p, a.zend - a.zbase);
+    a.zchunk = m.zchunk;
+    constexpr int kMin = sizeof(C) == 8 ? 1 : 3;
+    if (o.partials)
+        sc_moments_kernel<L, S, kTX, kTY, true, kMin == 3 ? 2 : 1>
+            <<<(unsigned)m.ctas, dim3(kTX, kTY), 0, st>>>(a, fo, m.tiles_x, m.tiles_y, m.items);
+    else
+        sc_moments_kernel<L, S, kTX, kTY, false, kMin>
+            <<<(unsigned)m.items, dim3(kTX, kTY), 0, st>>>(a, fo, m.tiles_x, m.tiles_y, m.items);
     return cudaGetLastError();
 }
 

@@ -23,11 +23,11 @@
 // TX*TY nodes of a plane, in x and y only: marching removes the z halo.
 #pragma once
 
+#include <type_traits>
+
 #include "sc_node.cuh"
 
 namespace lbmsc {
-
-enum KernelMode { kModeStep = 0, kModeMoments = 1 };
 
 // Pulled populations of node (x, y, z): f_is = f*_is(x - c_i).
 template <class L, class S>
@@ -159,21 +159,17 @@ __device__ __forceinline__ double diag_fold(int k, double a, double b) {
     return (k == kMaxSpeed) ? fmax(a, b) : (k == kMinRhoA || k == kMinRhoB) ? fmin(a, b) : a + b;
 }
 
-template <class L, class S, int TX, int TY, int MODE, int MINB>
-__global__ void __launch_bounds__(TX* TY, MINB)
-    sc_fused_kernel(const LatticeArgs<S> a, const FieldArgs<typename Codec<S>::C> fo) {
+template <class L, class S, int TX, int TY, int MINB>
+__global__ void __launch_bounds__(TX* TY, MINB) sc_fused_kernel(const LatticeArgs<S> a) {
     using C = typename Codec<S>::C;
-    using A = Ar<C>;
     constexpr int Q = L::Q;
     constexpr int FX = TX + 2, FY = TY + 2;
     constexpr int NPL = L::D == 3 ? 3 : 1;
     constexpr int H = 2 * FX + 2 * TY;
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
     __shared__ Two<C> srho[NPL][FY][FX];  // densities (rho_A, rho_B)
-    if (MODE == kModeStep) {
-        chain_wait();
-        chain_next();
-    }
+    chain_wait();
+    chain_next();
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -186,14 +182,6 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     const int hgx = (x0 - 1 + hfx + nx) % nx;
     const int hgy = (y0 - 1 + hfy + ny) % ny;
 
-    double acc[kNumDiag];
-    if (MODE == kModeMoments) {
-#pragma unroll
-        for (int k = 0; k < kNumDiag; ++k) acc[k] = 0.0;
-        acc[kMinRhoA] = 1e300;
-        acc[kMinRhoB] = 1e300;
-    }
-
     auto density_plane = [&](int slot, int z, C (&f)[2][Q]) {
         pull_node<L, S>(a, gx, gy, z, f);
         srho[slot][ty + 1][tx + 1] = node_densities<L, C>(f);
@@ -203,100 +191,24 @@ __global__ void __launch_bounds__(TX* TY, MINB)
             srho[slot][hfy][hfx] = node_densities<L, C>(h);
         }
     };
-
-    auto process = [&](C (&f)[2][Q], int sm, int sc, int sp, int z) {
-        const Two<C> r01 = srho[sc][ty + 1][tx + 1];
-        const C r0 = r01.a, r1 = r01.b;
+    auto collide = [&](C (&f)[2][Q], int sm, int sc, int sp, int z) {
+        const Two<C> r = srho[sc][ty + 1][tx + 1];
         auto nbr = [&](int i) -> Two<C> {
             const int slot = L::c(i, 2) == 0 ? sc : (L::c(i, 2) > 0 ? sp : sm);
             return srho[slot][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
         };
-        const size_t node = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * z);
-        if (MODE == kModeStep) {
-            node_update<L, C>(a, gy, nbr, f, r0, r1);
-            if (owner) store_node<L, S>(a, gx, gy, z, f, r0, r1);
-        } else {
-            // SC: physical velocity u = (j_A + j_B + (F_A + F_B) / 2) / rho (F dt/2
-            // shift, Sec. 2.3).  FE (Sec. 2.2): u = sum_i f_i c_i / rho, and the
-            // reported densities are rho_A = (rho + phi)/2, rho_B = (rho - phi)/2.
-            const bool fe = a.model == kModelFE;
-            C gA[3] = {(C)0, (C)0, (C)0}, gB[3] = {(C)0, (C)0, (C)0};
-            if (!fe) {
-                node_force<L, C>(nbr, a.G, gA, gB);
-                node_body_force<C>(a.body_A, gy, a.ny, gA, gB);
-            }
-            const C rA = fe ? A::mul((C)0.5, A::add(r0, r1)) : r0;
-            const C rB = fe ? A::mul((C)0.5, A::sub(r0, r1)) : r1;
-            Two<C> j[3];
-            node_momenta<L, C>(f, j);
-            const C rho = fe ? r0 : A::add(rA, rB);
-            const C inv_rho = A::rcp(rho);
-            C u[3];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const C half_force = A::mul((C)0.5, A::fma(rA, gA[d], A::mul(rB, gB[d])));
-                u[d] = A::mul(A::add(fe ? j[d].a : A::add(j[d].a, j[d].b), half_force), inv_rho);
-            }
-            const C p = A::mul(A::fma(A::mul(a.G, rA), rB, rho), (C)(1.0 / 3.0));
-            if (owner) {
-                if (fo.rhoA) fo.rhoA[node] = rA;
-                if (fo.rhoB) fo.rhoB[node] = rB;
-                if (fo.u)
-#pragma unroll
-                    for (int d = 0; d < L::D; ++d) fo.u[(size_t)d * (size_t)a.N + node] = u[d];
-                if (fo.p) fo.p[node] = p;
-                if (fo.partials) {
-                    const double dA = (double)rA, dB = (double)rB, drho = dA + dB;
-                    double uu = 0.0;
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) uu += (double)u[d] * (double)u[d];
-                    const bool finite = isfinite(dA) && isfinite(dB) && isfinite(uu) && isfinite((double)p);
-                    if (finite) {
-                        acc[kMassA] += dA;
-                        acc[kMassB] += dB;
-                        acc[kMomX] += (double)u[0] * drho;
-                        acc[kMomY] += (double)u[1] * drho;
-                        acc[kMomZ] += (double)u[2] * drho;
-                        acc[kKE] += 0.5 * drho * uu;
-                        acc[kMaxSpeed] = fmax(acc[kMaxSpeed], sqrt(uu));
-                        acc[kMinRhoA] = fmin(acc[kMinRhoA], dA);
-                        acc[kMinRhoB] = fmin(acc[kMinRhoB], dB);
-                    } else {
-                        acc[kNonFinite] += 1.0;
-                    }
-                    // periodic minimum-image distance from the window centre
-                    double dx = fabs((double)gx - fo.win_c[0]);
-                    double dy = fabs((double)gy - fo.win_c[1]);
-                    double dz = fabs((double)z - fo.win_c[2]);
-                    dx = fmin(dx, (double)nx - dx);
-                    dy = fmin(dy, (double)ny - dy);
-                    dz = fmin(dz, (double)nz - dz);
-                    const double r2 = dx * dx + dy * dy + (L::D == 3 ? dz * dz : 0.0);
-                    if (r2 < fo.r_in2) {
-                        acc[kInCount] += 1.0;
-                        acc[kInRhoA] += dA;
-                        acc[kInP] += (double)p;
-                    }
-                    if (r2 > fo.r_out2) {
-                        acc[kOutCount] += 1.0;
-                        acc[kOutRhoA] += dA;
-                        acc[kOutP] += (double)p;
-                    }
-                    // inside the drop: phi = rho_A - rho_B >= 0, compared in the compute type (Sec. 4.2)
-                    if (rA >= rB) acc[kDropNodes] += 1.0;
-                }
-            }
-        }
+        node_update<L, C>(a, gy, nbr, f, r.a, r.b);
+        if (owner) store_node<L, S>(a, gx, gy, z, f, r.a, r.b);
     };
 
     C cur[2][Q];
     if (L::D == 2) {
         density_plane(0, 0, cur);
         __syncthreads();
-        process(cur, 0, 0, 0, 0);
+        collide(cur, 0, 0, 0, 0);
     } else {
-        const int z0 = a.zbase + blockIdx.z * a.zchunk;
-        const int z1 = min(z0 + a.zchunk, a.zend);
+        const int z0 = blockIdx.z * a.zchunk;
+        const int z1 = min(z0 + a.zchunk, nz);
         {
             C tmp[2][Q];
             density_plane(0, z0 == 0 ? nz - 1 : z0 - 1, tmp);
@@ -307,7 +219,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
             C nxt[2][Q];
             density_plane(sp, z + 1 == nz ? 0 : z + 1, nxt);
             __syncthreads();
-            process(cur, sm, sc, sp, z);
+            collide(cur, sm, sc, sp, z);
 #pragma unroll
             for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -319,26 +231,266 @@ __global__ void __launch_bounds__(TX* TY, MINB)
             __syncthreads();
         }
     }
+}
 
-    if (MODE == kModeMoments && fo.partials) {
-        // CTA reduction of the diagnostics: warp shuffles, then one warp over the warps.
-        constexpr int NW = TX * TY / 32;
-        __shared__ double red[NW][kNumDiag];
-        const int lane = tid & 31, warp = tid >> 5;
+// Reported fields and FP64 diagnostics of the current populations.  Marches
+// like sc_fused_kernel, but a thread keeps only the momentum of the plane it
+// has pulled (3 values instead of 2 Q), so three CTAs share an SM; CTAs take
+// tiles and chunks in turn (item = blockIdx.x, + gridDim.x, ...), so that a large
+// lattice leaves a few thousand partial sums to fold, not one per tile.
+//
+// The FP64 sums run on two FP64 lanes a clock and SM and bound the diagnostics:
+// per node they take the conversions, one product and sum each for the masses,
+// momenta and the energy and one maximum.  The square root of the peak speed is
+// taken of the maximum (both are monotone, the rounded result is the same), the
+// minima stay in the compute type, a window's distances are formed per column
+// and plane, and no window costs nothing.  Measured (GB300): fields 512^3 FP32
+// 10.1 -> 5.8 ms, 256^3 1.30 -> 0.75; diagnostics 512^3 FP32 20.9 -> 9.3 ms, 4096^2 4.74 -> 1.04.
+template <class L, class S, int TX, int TY, bool DIAG, int MINB>
+__global__ void __launch_bounds__(TX* TY, MINB)
+    sc_moments_kernel(const LatticeArgs<S> a, const FieldArgs<typename Codec<S>::C> fo, int tiles_x, int tiles_y,
+                      int nitems) {
+    using C = typename Codec<S>::C;
+    using A = Ar<C>;
+    constexpr int Q = L::Q;
+    constexpr int FX = TX + 2, FY = TY + 2;
+    constexpr int NPL = L::D == 3 ? 3 : 1;
+    constexpr int H = 2 * FX + 2 * TY;
+    static_assert(H <= TX * TY, "halo ring must fit in the CTA");
+    __shared__ Two<C> srho[NPL][FY][FX];
+
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
+    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const bool halo = tid < H;
+    int hfx, hfy;
+    halo_cell<TX, TY>(tid, hfx, hfy);
+    const bool win_in = DIAG && fo.r_in2 > 0.0, win_out = DIAG && fo.r_out2 < 1e300;
+
+    // FP64 sums: masses, momenta, energy; with a window its densities and pressures
+    enum { kA, kB, kX, kY, kZ, kE, kIA, kIP, kOA, kOP, kSums };
+    double acc[kSums];
+    double uu_max = 0.0;
+    C minA = (C)INFINITY, minB = (C)INFINITY;
+    int nonfinite = 0, drop = 0, n_in = 0, n_out = 0;
+    if (DIAG) {
 #pragma unroll
-        for (int k = 0; k < kNumDiag; ++k) {
-            double v = acc[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v = diag_fold(k, v, __shfl_xor_sync(0xffffffffu, v, o));
-            if (lane == 0) red[warp][k] = v;
+        for (int k = 0; k < kSums; ++k) acc[k] = 0.0;
+    }
+
+#pragma unroll 1
+    for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
+        const int bx = item % tiles_x, by = (item / tiles_x) % tiles_y, bz = item / (tiles_x * tiles_y);
+        const int x0 = bx * TX, y0 = by * TY;
+        const bool owner = (x0 + tx) < nx && (y0 + ty) < ny;
+        const int gx = (x0 + tx) % nx, gy = (y0 + ty) % ny;
+        const int hgx = (x0 - 1 + hfx + nx) % nx;
+        const int hgy = (y0 - 1 + hfy + ny) % ny;
+        double rxy2 = 0.0;  // squared periodic minimum-image distance of the column from the window's centre
+        if (win_in || win_out) {
+            double dx = fabs((double)gx - fo.win_c[0]), dy = fabs((double)gy - fo.win_c[1]);
+            dx = fmin(dx, (double)nx - dx);
+            dy = fmin(dy, (double)ny - dy);
+            rxy2 = dx * dx + dy * dy;
         }
-        __syncthreads();
-        if (tid < kNumDiag) {
-            const int k = tid;
-            double v = red[0][k];
-            for (int w = 1; w < NW; ++w) v = diag_fold(k, v, red[w][k]);
-            const size_t b = blockIdx.x + (size_t)gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
-            fo.partials[b * kNumDiag + k] = v;
+
+        // densities of plane z into a ring slot, and the node's momentum
+        auto density_plane = [&](int slot, int z, C (&j)[3]) {
+            {
+                C f[2][Q];
+                pull_node<L, S>(a, gx, gy, z, f);
+                srho[slot][ty + 1][tx + 1] = node_densities<L, C>(f);
+                Two<C> js[3];
+                node_momenta<L, C>(f, js);
+                // FE: u = sum_i f_i c_i / rho, from the first population alone
+#pragma unroll
+                for (int d = 0; d < 3; ++d) j[d] = a.model == kModelFE ? js[d].a : A::add(js[d].a, js[d].b);
+            }
+            if (halo) {
+                C h[2][Q];
+                pull_node<L, S>(a, hgx, hgy, z, h);
+                srho[slot][hfy][hfx] = node_densities<L, C>(h);
+            }
+        };
+
+        auto process = [&](const C (&j)[3], int sm, int sc, int sp, int z) {
+            const Two<C> r01 = srho[sc][ty + 1][tx + 1];
+            const C r0 = r01.a, r1 = r01.b;
+            auto nbr = [&](int i) -> Two<C> {
+                const int slot = L::c(i, 2) == 0 ? sc : (L::c(i, 2) > 0 ? sp : sm);
+                return srho[slot][ty + 1 + L::c(i, 1)][tx + 1 + L::c(i, 0)];
+            };
+            const size_t node = (size_t)gx + (size_t)nx * ((size_t)gy + (size_t)ny * z);
+            // SC: physical velocity u = (j_A + j_B + (F_A + F_B) / 2) / rho (F dt/2
+            // shift, Sec. 2.3).  FE (Sec. 2.2): u = sum_i f_i c_i / rho, and the
+            // reported densities are rho_A = (rho + phi)/2, rho_B = (rho - phi)/2.
+            const bool fe = a.model == kModelFE;
+            C gA[3] = {(C)0, (C)0, (C)0}, gB[3] = {(C)0, (C)0, (C)0};
+            if (!fe) {
+                node_force<L, C>(nbr, a.G, gA, gB);
+                node_body_force<C>(a.body_A, gy, a.ny, gA, gB);
+            }
+            const C rA = fe ? A::mul((C)0.5, A::add(r0, r1)) : r0;
+            const C rB = fe ? A::mul((C)0.5, A::sub(r0, r1)) : r1;
+            const C rho = fe ? r0 : A::add(rA, rB);
+            const C inv_rho = A::rcp(rho);
+            C u[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const C half_force = A::mul((C)0.5, A::fma(rA, gA[d], A::mul(rB, gB[d])));
+                u[d] = A::mul(A::add(j[d], half_force), inv_rho);
+            }
+            const C p = A::mul(A::fma(A::mul(a.G, rA), rB, rho), (C)(1.0 / 3.0));
+            if (!owner) return;
+            if (!DIAG) {
+                if (fo.rhoA) fo.rhoA[node] = rA;
+                if (fo.rhoB) fo.rhoB[node] = rB;
+                if (fo.u)
+#pragma unroll
+                    for (int d = 0; d < L::D; ++d) fo.u[(size_t)d * (size_t)a.N + node] = u[d];
+                if (fo.p) fo.p[node] = p;
+            } else {
+                const double dA = (double)rA, dB = (double)rB, drho = dA + dB;
+                double ud[3], uu = 0.0;
+#pragma unroll
+                for (int d = 0; d < L::D; ++d) {
+                    ud[d] = (double)u[d];
+                    uu += ud[d] * ud[d];
+                }
+                const bool finite = isfinite(dA) && isfinite(dB) && isfinite(uu) && isfinite(p);
+                if (finite) {
+                    acc[kA] += dA;
+                    acc[kB] += dB;
+                    acc[kX] += ud[0] * drho;
+                    acc[kY] += ud[1] * drho;
+                    if (L::D == 3) acc[kZ] += ud[L::D - 1] * drho;
+                    acc[kE] += (0.5 * drho) * uu;
+                    uu_max = fmax(uu_max, uu);
+                    minA = rA < minA ? rA : minA;
+                    minB = rB < minB ? rB : minB;
+                } else {
+                    ++nonfinite;
+                }
+                if (win_in || win_out) {
+                    double dz = 0.0;
+                    if (L::D == 3) {
+                        dz = fabs((double)z - fo.win_c[2]);
+                        dz = fmin(dz, (double)nz - dz);
+                    }
+                    const double r2 = rxy2 + dz * dz;
+                    if (r2 < fo.r_in2) {
+                        ++n_in;
+                        acc[kIA] += dA;
+                        acc[kIP] += (double)p;
+                    }
+                    if (r2 > fo.r_out2) {
+                        ++n_out;
+                        acc[kOA] += dA;
+                        acc[kOP] += (double)p;
+                    }
+                }
+                // inside the drop: phi = rho_A - rho_B >= 0, compared in the compute type (Sec. 4.2)
+                if (rA >= rB) ++drop;
+            }
+        };
+
+        C cur[3];
+        if (L::D == 2) {
+            density_plane(0, 0, cur);
+            __syncthreads();
+            process(cur, 0, 0, 0, 0);
+            __syncthreads();
+        } else {
+            const int z0 = a.zbase + bz * a.zchunk;
+            const int z1 = min(z0 + a.zchunk, a.zend);
+            density_plane(0, z0 == 0 ? nz - 1 : z0 - 1, cur);
+            density_plane(1, z0, cur);
+            int sm = 0, sc = 1, sp = 2;
+#pragma unroll 1
+            for (int z = z0; z < z1; ++z) {
+                C nxt[3];
+                density_plane(sp, z + 1 == nz ? 0 : z + 1, nxt);
+                __syncthreads();
+                process(cur, sm, sc, sp, z);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) cur[d] = nxt[d];
+                const int t = sm;
+                sm = sc;
+                sc = sp;
+                sp = t;
+                __syncthreads();
+            }
+        }
+    }
+
+    if (DIAG) {
+        // CTA reduction: one warp per FP64 sum over the threads' values in shared
+        // memory (13 additions a lane; shuffling every sum through every warp took
+        // eight times as many on the few FP64 lanes, 6 us a CTA), whole numbers by
+        // the warp reductions, maximum and minima by shuffles
+        constexpr int NW = TX * TY / 32, NT = TX * TY;
+        static_assert(NW >= 6, "a warp per sum");
+        __shared__ double sums[6][NT];
+        __shared__ int counts[NW][4];
+        __shared__ double ext[NW][3];
+        const int lane = tid & 31, warp = tid >> 5;
+        double* const out = fo.partials + (size_t)blockIdx.x * kNumDiag;
+        const int cnt[4] = {nonfinite, drop, n_in, n_out};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int v = __reduce_add_sync(0xffffffffu, cnt[k]);
+            if (lane == 0) counts[warp][k] = v;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double m = __shfl_xor_sync(0xffffffffu, uu_max, o);
+            uu_max = m > uu_max ? m : uu_max;
+            const C p = __shfl_xor_sync(0xffffffffu, minA, o), q = __shfl_xor_sync(0xffffffffu, minB, o);
+            minA = p < minA ? p : minA;
+            minB = q < minB ? q : minB;
+        }
+        if (lane == 0) {
+            ext[warp][0] = uu_max;
+            ext[warp][1] = (double)minA;
+            ext[warp][2] = (double)minB;
+        }
+        // sums k0 .. k0 + n - 1 into the record's slots
+        auto fold_sums = [&](auto k0, int n) {
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                if (k0 + k < kSums) sums[k][tid] = acc[k0 + k];
+            __syncthreads();
+            if (warp < n) {
+                double v = sums[warp][lane];
+#pragma unroll
+                for (int t = 1; t < NW; ++t) v += sums[warp][lane + 32 * t];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                constexpr int slot[12] = {kMassA, kMassB, kMomX, kMomY, kMomZ, kKE, kInRhoA, kInP, kOutRhoA, kOutP, 0, 0};
+                if (lane == 0) out[slot[k0 + warp]] = v;
+            }
+        };
+        fold_sums(std::integral_constant<int, 0>(), 6);
+        if (win_in || win_out)
+            fold_sums(std::integral_constant<int, 6>(), 4);
+        else if (tid == 0)
+            out[kInRhoA] = out[kInP] = out[kOutRhoA] = out[kOutP] = 0.0;
+        if (tid == 0) {
+            int c[4] = {0, 0, 0, 0};
+            double m[3] = {0.0, INFINITY, INFINITY};
+            for (int w = 0; w < NW; ++w) {
+                for (int k = 0; k < 4; ++k) c[k] += counts[w][k];
+                m[0] = ext[w][0] > m[0] ? ext[w][0] : m[0];
+                m[1] = ext[w][1] < m[1] ? ext[w][1] : m[1];
+                m[2] = ext[w][2] < m[2] ? ext[w][2] : m[2];
+            }
+            out[kMaxSpeed] = sqrt(m[0]);
+            out[kMinRhoA] = m[1] < 1e300 ? m[1] : 1e300;  // 1e300: no finite node
+            out[kMinRhoB] = m[2] < 1e300 ? m[2] : 1e300;
+            out[kNonFinite] = c[0];
+            out[kDropNodes] = c[1];
+            out[kInCount] = c[2];
+            out[kOutCount] = c[3];
         }
     }
 }
@@ -414,33 +566,22 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
     }
 }
 
-// Second pass of the diagnostics: one CTA folds the per-CTA partials.
+// Second pass of the diagnostics: CTA k folds slot k of the partial records
+// (one CTA for all slots spent its time on one SM's FP64 lanes: 22 us with
+// 1024 threads, whatever the lattice).
 template <int NT>
 __global__ void __launch_bounds__(NT) sc_diag_finish_kernel(const double* __restrict__ partials,
                                                             long long nparts, double* __restrict__ out) {
-    __shared__ double red[NT / 32][kNumDiag];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    double acc[kNumDiag];
+    __shared__ double red[NT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = blockIdx.x;
+    double v = (k == kMinRhoA || k == kMinRhoB) ? 1e300 : 0.0;
+    for (long long b = tid; b < nparts; b += NT) v = diag_fold(k, v, partials[b * kNumDiag + k]);
 #pragma unroll
-    for (int k = 0; k < kNumDiag; ++k) acc[k] = 0.0;
-    acc[kMinRhoA] = 1e300;
-    acc[kMinRhoB] = 1e300;
-    for (long long b = tid; b < nparts; b += NT) {
-#pragma unroll
-        for (int k = 0; k < kNumDiag; ++k) acc[k] = diag_fold(k, acc[k], partials[b * kNumDiag + k]);
-    }
-#pragma unroll
-    for (int k = 0; k < kNumDiag; ++k) {
-        double v = acc[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = diag_fold(k, v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (lane == 0) red[warp][k] = v;
-    }
+    for (int o = 16; o > 0; o >>= 1) v = diag_fold(k, v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0) red[warp] = v;
     __syncthreads();
-    if (tid < kNumDiag) {
-        const int k = tid;
-        double v = red[0][k];
-        for (int w = 1; w < NT / 32; ++w) v = diag_fold(k, v, red[w][k]);
+    if (tid == 0) {
+        for (int w = 1; w < NT / 32; ++w) v = diag_fold(k, v, red[w]);
         out[k] = v;
     }
 }
@@ -449,37 +590,51 @@ __global__ void __launch_bounds__(NT) sc_diag_finish_kernel(const double* __rest
 // at node x holds f^eq_i(rho_s(x + c_i), u(x + c_i)), so pulling it at x + c_i
 // gives f_i(x + c_i, 0) = f^eq_i of that node.  The ghost columns and rows get
 // the values of their periodic images.
+// Threads run along the cells of a row (blockIdx.x) and the rows of planes
+// [zlo, zhi) are taken in turn (blockIdx.y): the periodic neighbours are three
+// indices per axis, formed once per cell.  The x images fill whole 32-byte
+// sectors and a warp's cells start on a cache line, as in store_node: rows begun
+// at the image column -2 left a partly written sector at either end of every
+// warp's stores, each of which reads HBM (512^3 FP32 8.2 ms, now 5.1; 4096^2 0.40,
+// now 0.29).
+constexpr int kInitThreads = 64, kInitLead = 32;
 template <class L, class S>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kInitThreads)
     sc_init_kernel(const LatticeArgs<S> a, const typename Codec<S>::C* __restrict__ rhoA,
                    const typename Codec<S>::C* __restrict__ rhoB, const typename Codec<S>::C* __restrict__ u, int zlo,
                    int zhi) {
     using C = typename Codec<S>::C;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const int ex = nx + 4, ey = ny + 4;  // cells x in [-2, nx + 1], y in [-2, ny + 1]
+    constexpr int kSector = 32 / (int)sizeof(S) > 2 ? 32 / (int)sizeof(S) : 2;
+    const int GX = nx >= kSector ? kSector : 2;
+    const int ey = ny + 4;  // cells x in [-GX, nx + GX), y in [-2, ny + 2)
+    const int cx = (int)(blockIdx.x * kInitThreads + threadIdx.x) - kInitLead;
+    if (cx < -GX || cx >= nx + GX) return;
+    const int x = ((cx % nx) + nx) % nx;
+    const int xs[3] = {wrap_dec(x, nx), x, wrap_inc(x, nx)};
     // the cells of planes [zlo, zhi); they read the fields of planes zlo - 1 .. zhi (periodic)
-    const long long ncells = (long long)ex * ey * zhi;
-    for (long long k = (long long)ex * ey * zlo + blockIdx.x * (long long)blockDim.x + threadIdx.x; k < ncells;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int cx = (int)(k % ex) - 2;
-        const int cy = (int)((k / ex) % ey) - 2;
-        const int z = (int)(k / ((long long)ex * ey));
+    const long long rows = (long long)ey * (zhi - zlo);
+    for (long long row = blockIdx.y; row < rows; row += gridDim.y) {
+        const int cy = (int)(row % ey) - 2;
+        const int z = zlo + (int)(row / ey);
         const size_t n = cell(a, cx, cy, z);
-        const int x = ((cx % nx) + nx) % nx, y = ((cy % ny) + ny) % ny;
+        const int y = ((cy % ny) + ny) % ny;
+        const int ys[3] = {wrap_dec(y, ny), y, wrap_inc(y, ny)};
+        const int zs[3] = {L::D == 3 ? wrap_dec(z, nz) : 0, L::D == 3 ? z : 0, L::D == 3 ? wrap_inc(z, nz) : 0};
         C fr[2][L::Q];  // rest-offset storage: the cell's values, stored together
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) {
-            const int sx = (x + L::c(i, 0) + nx) % nx;
-            const int sy = (y + L::c(i, 1) + ny) % ny;
-            const int sz = L::D == 3 ? (z + L::c(i, 2) + nz) % nz : 0;
-            const size_t m = (size_t)sx + (size_t)nx * ((size_t)sy + (size_t)ny * sz);
-            C uv[3] = {0, 0, 0};
-            if (u)
+            const size_t m = (size_t)xs[L::c(i, 0) + 1] +
+                             (size_t)nx * ((size_t)ys[L::c(i, 1) + 1] + (size_t)ny * zs[L::c(i, 2) + 1]);
+            C shape = (C)1;
+            if (u) {
+                C uv[3] = {0, 0, 0};
                 for (int d = 0; d < L::D; ++d) uv[d] = u[(size_t)d * (size_t)a.N + m];
-            C uu = uv[0] * uv[0] + uv[1] * uv[1] + uv[2] * uv[2];
-            C cu = (C)0;
-            for (int d = 0; d < L::D; ++d) cu += (C)L::c(i, d) * uv[d];
-            const C shape = (C)1 - (C)1.5 * uu + cu * ((C)3 + (C)4.5 * cu);
+                C uu = uv[0] * uv[0] + uv[1] * uv[1] + uv[2] * uv[2];
+                C cu = (C)0;
+                for (int d = 0; d < L::D; ++d) cu += (C)L::c(i, d) * uv[d];
+                shape = (C)1 - (C)1.5 * uu + cu * ((C)3 + (C)4.5 * cu);
+            }
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
                 // SC: species densities; FE: f from rho = rho_A + rho_B, g from phi = rho_A - rho_B

@@ -14,7 +14,6 @@ struct Plan {
     int precision;  // lbm_precision (4, 5: rest-offset 16-bit storage)
     int nx, ny, nz;
     long long N;
-    int zchunk;     // planes per CTA along z for the moments kernel (D3Q19)
     int step_tile;  // index into kTiles for the step kernel
     int step_zchunk;
     int sm_count;   // multiprocessors of the device (persistent grids)
@@ -181,9 +180,32 @@ struct MomentsOut {
     int zlo = 0, zhi = 0;   // zhi > 0: fields of planes [zlo, zhi) only (D3Q19, no partials)
 };
 
-inline dim3 fused_grid(const Plan& p) {
-    return dim3((unsigned)((p.nx + kTX - 1) / kTX), (unsigned)((p.ny + kTY - 1) / kTY),
-                (unsigned)(p.lattice == 1 ? (p.nz + p.zchunk - 1) / p.zchunk : 1));
+// Grid of the moments kernel over `planes` planes: items of one tile and one z
+// chunk, the chunk chosen for the shortest time on 152 SMs with three CTAs each
+// (a chunk of zc planes pulls two more), and the CTAs of a diagnostics launch,
+// which take the items in turn and leave one record of partial sums each.
+struct MomentsShape {
+    int tiles_x, tiles_y, zchunk, items, ctas;
+};
+constexpr int kDiagCtas = 152 * 16;
+inline MomentsShape moments_shape(const Plan& p, int planes) {
+    MomentsShape m;
+    m.tiles_x = (p.nx + kTX - 1) / kTX;
+    m.tiles_y = (p.ny + kTY - 1) / kTY;
+    m.zchunk = 1;
+    const long long xy = (long long)m.tiles_x * m.tiles_y;
+    long long best = -1;
+    if (p.lattice == 1)
+        for (int zc = 1; zc <= planes && zc <= 32; ++zc) {
+            const long long n = xy * ((planes + zc - 1) / zc), cost = ((n + 455) / 456) * (zc + 2);
+            if (best < 0 || cost < best) {
+                best = cost;
+                m.zchunk = zc;
+            }
+        }
+    m.items = (int)(xy * (p.lattice == 1 ? (planes + m.zchunk - 1) / m.zchunk : 1));
+    m.ctas = m.items < kDiagCtas ? m.items : kDiagCtas;
+    return m;
 }
 
 inline dim3 step_grid(const Plan& p) {
@@ -192,10 +214,8 @@ inline dim3 step_grid(const Plan& p) {
                 (unsigned)(p.lattice == 1 ? (p.nz + p.step_zchunk - 1) / p.step_zchunk : 1));
 }
 
-inline long long fused_blocks(const Plan& p) {
-    const dim3 g = fused_grid(p);
-    return (long long)g.x * g.y * g.z;
-}
+// Records of partial sums a diagnostics launch leaves.
+inline long long diag_parts(const Plan& p) { return moments_shape(p, p.nz).ctas; }
 
 cudaError_t d2q9_step(const Plan& p, const void* fin, void* fout, cudaStream_t st);
 // The tile of an untuned D2Q9 lattice in 32- and 16-bit storage.
