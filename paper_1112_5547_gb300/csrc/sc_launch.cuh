@@ -208,6 +208,15 @@ inline MomentsShape moments_shape(const Plan& p, int planes) {
     return m;
 }
 
+// Columns of tile 3 in FP64 on a D3Q19 lattice: 16x8 where that covers fewer
+// columns outside the lattice than 32x4.
+inline void f64_tile3(const Plan& p, int& tx, int& ty) {
+    const long long wide = (long long)((p.nx + 31) / 32 * 32) * ((p.ny + 3) / 4 * 4);
+    const long long high = (long long)((p.nx + 15) / 16 * 16) * ((p.ny + 7) / 8 * 8);
+    tx = high < wide ? 16 : 32;
+    ty = high < wide ? 8 : 4;
+}
+
 inline dim3 step_grid(const Plan& p) {
     const TileShape t = kTiles[p.step_tile];
     return dim3((unsigned)((p.nx + t.tx - 1) / t.tx), (unsigned)((p.ny + t.ty - 1) / t.ty),

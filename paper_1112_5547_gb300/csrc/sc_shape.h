@@ -12,7 +12,7 @@
 // 13: 168 (43), 16: 194 (52), 20: 173 (42), 28: 220 (58), 43: 193 (44 and the
 // one-wave penalty)).  At least 16 planes a chunk on one tile for every lattice,
 // the rule before, gave 313 us there, 18.5 ms instead of 7.1 at 512^3, 84 us
-// instead of 7.4 at 32^3 and 562 instead of 143 at 48^3 in FP64.
+// instead of 7.4 at 32^3 and 562 instead of 98 at 48^3 in FP64.
 #pragma once
 
 #include "sc_launch.cuh"
@@ -70,7 +70,8 @@ inline StepModel step_model(const Plan& p, int tile) {
 
 // Time of a step in plane times of the 64x6 tile.
 inline double step_cost(const Plan& p, int tile, int zc) {
-    const TileShape& t = kTiles[tile];
+    TileShape t = kTiles[tile];
+    if (p.precision == 0 && tile == 3) f64_tile3(p, t.tx, t.ty);
     const StepModel m = step_model(p, tile);
     const long long xy = (long long)((p.nx + t.tx - 1) / t.tx) * ((p.ny + t.ty - 1) / t.ty);
     const long long slots = (long long)m.per_sm * p.sm_count, full = xy * (p.nz / zc);
@@ -98,9 +99,10 @@ inline double step_cost(const Plan& p, int tile, int zc) {
     const double n = (double)(full + (last ? xy : 0)) / (double)slots;  // waves
     double f = m.weight;
     if (p.precision == 0) {
-        // all CTAs are resident early and share their SM's units: the time is the
-        // work of the SM that gets the first CTA of every round; one CTA alone
-        // on an SM loses a fifth of the rate
+        // CTAs are resident early and share their SM's units: the time is the work
+        // of the SM that gets the first CTA of every round (96^3: 24 planes a chunk
+        // 701 us, 20 with a short last chunk 946); one CTA alone on an SM loses a
+        // fifth of the rate
         const long long rounds = (full + (last ? xy : 0) + slots - 1) / slots, rfull = (full + slots - 1) / slots;
         end = (double)rfull * a + (double)(rounds - rfull) * b;
         if (n <= 1.0) f *= 1.2;
@@ -126,7 +128,7 @@ inline int best_zchunk(const Plan& p, int tile, double* cost = nullptr) {
     double c = step_cost(p, tile, 1);
     for (int z = 2; z <= p.nz && z <= most; ++z) {
         const double k = step_cost(p, tile, z);
-        if (k < c * (1.0 - 1e-9)) {
+        if (k < c * (p.precision == 0 ? 1.0 + 1e-9 : 1.0 - 1e-9)) {  // FP64: the longer of equals
             c = k;
             best = z;
         }
