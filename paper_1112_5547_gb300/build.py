@@ -49,7 +49,7 @@ def up_to_date() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(PFM_LIB):
         return False
     t = min(os.path.getmtime(LIB), os.path.getmtime(PFM_LIB))
-    deps = _deps() + sorted(glob.glob(os.path.join(PFM_CSRC, "*.cu"))) + [os.path.join(ROOT, "include", "pfm.h")]
+    deps = _deps() + sorted(glob.glob(os.path.join(PFM_CSRC, "*.cu*"))) + [os.path.join(ROOT, "include", "pfm.h")]
     return all(os.path.getmtime(d) <= t for d in deps)
 
 
