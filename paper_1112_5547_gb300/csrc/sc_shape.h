@@ -118,15 +118,22 @@ inline double step_cost(const Plan& p, int tile, int zc) {
     return end * f + m.launch;
 }
 
+constexpr int kMaxGridYZ = 65535;
+
+// Whether the tile rows of a lattice fit the second dimension of a grid.
+inline bool rows_fit(int tile, const Plan& p) { return (p.ny + kTiles[tile].ty - 1) / kTiles[tile].ty <= kMaxGridYZ; }
+
 // Best z chunk of a tile (D3Q19).
 inline int best_zchunk(const Plan& p, int tile, double* cost = nullptr) {
     // long chunks let neighbouring tiles drift apart and lose the halo rows they
     // share in L2 (256^3 FP32, chunks of 24 / 43 / 64 planes: 1.05 / 1.14 / 1.19
     // ms; bf16 rest-offset 0.765 / 0.796 / 0.839)
-    const int most = p.precision >= 2 ? 48 : 32;
-    int best = 1;
-    double c = step_cost(p, tile, 1);
-    for (int z = 2; z <= p.nz && z <= most; ++z) {
+    const int least = (p.nz + kMaxGridYZ - 1) / kMaxGridYZ;  // chunks are a grid's third dimension
+    int most = p.precision >= 2 ? 48 : 32;
+    if (most < least) most = least;
+    int best = least;
+    double c = step_cost(p, tile, least);
+    for (int z = least + 1; z <= p.nz && z <= most; ++z) {
         const double k = step_cost(p, tile, z);
         if (k < c * (p.precision == 0 ? 1.0 + 1e-9 : 1.0 - 1e-9)) {  // FP64: the longer of equals
             c = k;
@@ -143,14 +150,14 @@ inline void pick_step(Plan& p) {
         // D2Q9: 32x4 tiles, four to six CTAs per SM (4096^2 FP32 0.461 ms a
         // step against 0.487 with 32x8, 64^2 2.7 us against 3.2); FP64 is
         // bound by its units and 32x8 has the smaller halo (256^2 30.5 / 31.2 us)
-        p.step_tile = p.precision == 0 ? 0 : kTileD2;
+        p.step_tile = p.precision == 0 || !rows_fit(kTileD2, p) ? 0 : kTileD2;
         p.step_zchunk = 1;
         return;
     }
     double best = 0.0;
     int tile = -1, zc = 1;
     for (const int* t = step_candidates(p); *t >= 0; ++t) {
-        if (!tile_fits(*t, p)) continue;
+        if (!tile_fits(*t, p) || !rows_fit(*t, p)) continue;
         double c;
         const int z = best_zchunk(p, *t, &c);
         if (tile < 0 || c < best * (1.0 - 1e-9)) {
@@ -159,7 +166,11 @@ inline void pick_step(Plan& p) {
             zc = z;
         }
     }
-    p.step_tile = tile;  // the register kernels at the end of each list fit every lattice
+    if (tile < 0) {  // more rows than any candidate's grid holds
+        tile = 0;
+        zc = best_zchunk(p, 0);
+    }
+    p.step_tile = tile;
     p.step_zchunk = zc;
 }
 

@@ -957,15 +957,6 @@ LBM_SC_API lbm_status pfm_create(const pfm_params* p, void* d_ws, size_t bytes, 
         return LBM_ERR_CUDA;
     }
     h->fused = fused_shape(g, dbl);
-    if (h->fused.ok) {
-        const int n[3] = {g.nx, g.ny, g.nz};
-        for (int a = 0; a < g.dim; ++a)
-            pfm_fft::twiddle_kernel<<<4, 256, 0, h->stream>>>((double2*)(h->ws + L.tw[a]), n[a]);
-        if (cudaGetLastError() != cudaSuccess) {
-            pfm_destroy(h);
-            return LBM_ERR_CUDA;
-        }
-    }
     *out = h;
     return LBM_OK;
 }
@@ -976,6 +967,12 @@ LBM_SC_API lbm_status pfm_init(pfm_handle* h, const void* d_phi, const void* d_u
     const int D = g.dim;
     const size_t rb = real_bytes(&h->params), cb = 2 * rb;
     unsigned char* w = h->ws;
+    if (h->fused.ok) {
+        const int n[3] = {g.nx, g.ny, g.nz};
+        for (int a = 0; a < D; ++a)
+            pfm_fft::twiddle_kernel<<<4, 256, 0, h->stream>>>((double2*)(w + h->L.tw[a]), n[a]);
+        if (cudaGetLastError() != cudaSuccess) return LBM_ERR_CUDA;
+    }
     // the forward batch's inputs: phi, u_a, the rest zero; transformed together
     if (cudaMemsetAsync(w + h->L.rphys, 0, n_forward(D) * g.nreal * rb, h->stream) != cudaSuccess) return LBM_ERR_CUDA;
     if (cudaMemcpyAsync(w + h->L.rphys, d_phi, g.nreal * rb, cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess)

@@ -39,6 +39,23 @@ def test_untuned_shape_is_one_the_library_accepts():
                     lib.lbm_sc_destroy(h)
 
 
+def test_untuned_shape_of_long_lattices_fits_a_grid():
+    """Tiles along y and chunks along z are grid dimensions of at most 65535."""
+    from paper_1112_5547_gb300 import build, lbm_sc as lib
+    build.build()
+    for lat, shape in ((0, (262140, 16)), (0, (262141, 16)), (0, (524280, 16)), (1, (1, 300000, 8)), (1, (2, 524280, 16)),
+                       (1, (65536, 8, 8)), (1, (2100000, 4, 4)), (1, (2100000, 8, 32))):
+        for prec in PRECISIONS:
+            p = lib.make_params(lat, shape, 1.0, 1.0, 2.0, prec)
+            h = lib.lbm_sc_create(p, 256 * 1024, lib.lbm_sc_workspace_bytes(p), 0)
+            try:
+                tile, zc = lib.lbm_sc_get_tuning(h)
+                assert -(-p.ny // lib.TILES[tile][1]) <= 65535
+                assert 1 <= zc <= p.nz and -(-p.nz // zc) <= 65535
+            finally:
+                lib.lbm_sc_destroy(h)
+
+
 def _run(lib, lat, shape, prec, kw, tuning, fields, steps):
     import torch
     ref = dict(rho_ref_A=0.5, rho_ref_B=0.5) if prec == "bf16" else {}
