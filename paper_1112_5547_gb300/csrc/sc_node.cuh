@@ -36,17 +36,10 @@
 
 namespace lbmsc {
 
-// rho = (f_1 + f_2 + ... + f_{Q-1}) + f_0, the moving populations first and
-// the rest population last, in one fixed order.  rho enters the equilibria
-// and the velocity; the closure of f^eq_0 below does not round through it.
-template <class L, class C> __device__ __forceinline__ C node_density(const C (&f)[L::Q]) {
-    C r = f[1];
-#pragma unroll
-    for (int i = 2; i < L::Q; ++i) r = Ar<C>::add(r, f[i]);
-    return Ar<C>::add(r, f[0]);
-}
-
-// The densities of both species, each summed as node_density sums it.
+// rho_s = (f_1 + f_2 + ... + f_{Q-1}) + f_0 of both species, the moving
+// populations first and the rest population last, in one fixed order.  rho enters
+// the equilibria and the velocity; the closure of f^eq_0 below does not round
+// through it.
 template <class L, class C> __device__ __forceinline__ Two<C> node_densities(const C (&f)[2][L::Q]) {
     Two<C> r{f[0][1], f[1][1]};
 #pragma unroll

@@ -202,7 +202,7 @@ __device__ __forceinline__ void tma_pulled_pair(const unsigned char* sb, int i, 
 
 // Density rho_s of frame node (fx, fy) for one species s (a run-time value:
 // the same instructions read the other species' planes or half-words), with
-// the values decoded and summed exactly as node_density sums a node's pulls
+// the values decoded and summed exactly as node_densities sums a node's pulls
 // (moving populations in order, the rest population last).
 template <int TX, int TY, int S, class St>
 __device__ __forceinline__ float tma_density(const unsigned char* sb, int s, int fx, int fy, float ref_s) {
