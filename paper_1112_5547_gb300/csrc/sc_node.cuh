@@ -242,56 +242,10 @@ __device__ __forceinline__ void node_relax(const F& f, V rho, const V (&u)[3], V
     f.set(0, A::fma(omega, neg2(neq.get()), f.get(0)));
 }
 
-// The same in FP64, in fewer operations: the FP64 units (two FMA a clock and
-// SM) bound every FP64 kernel, so opposite directions share the even part
-// e = w rho (1 - 3/2 u.u + 9/2 (c.u)^2) and the odd part o = 3 w rho c.u of their
-// equilibria, omega is folded into both, and the closure is the sum of the even
-// parts, f^eq_0 = rho - 2 sum e (rounding at the scale of rho is 1e-16 here; the
-// FP32 form above avoids it).  About 97 operations a species instead of 127 (GB300,
-// us a step: D2Q9 256^2 33 -> 28, with Guo forcing 43 -> 33; D3Q19 96^3 772 -> 701).
-// force (Guo) or null: the source's even and odd parts join e and o, see
-// node_relax_guo.
-template <class L, bool GUO>
-__device__ __forceinline__ void node_relax64(double (&f)[L::Q], double rho, const double (&u)[3],
-                                             const double (&force)[3], double omega) {
-    using A = Ar<double>;
-    static_assert(opposite_pairs<L>(), "velocity order must pair c_{i+1} = -c_i");
-    const double base = A::fma(-1.5, node_dot2<L, double>(u, u), 1.0);
-    const double keep = A::sub(1.0, omega), orho = A::mul(omega, rho);
-    const double ks = GUO ? A::fma(-0.5, omega, 1.0) : 0.0;  // 1 - 1 / (2 tau)
-    const double m3uF = GUO ? A::mul(-3.0, node_dot2<L, double>(u, force)) : 0.0;
-    SignedSum<double> even;
-#pragma unroll
-    for (int i = 1; i < L::Q; i += 2) {
-        const double w = L::w(i), wr = A::mul(w, orho);
-        const double cu = node_cu<L, double>(i, u);
-        double e = A::mul(wr, A::fma(A::mul(4.5, cu), cu, base));
-        double o = A::mul(A::mul(3.0, wr), cu);
-        if (GUO) {
-            const double cF = node_cu<L, double>(i, force), kw = A::mul(ks, w);
-            e = A::fma(kw, A::fma(A::mul(9.0, cu), cF, m3uF), e);
-            o = A::fma(A::mul(3.0, kw), cF, o);
-        }
-        even.add(e);
-        f[i] = A::fma(keep, f[i], A::add(e, o));
-        f[i + 1] = A::fma(keep, f[i + 1], A::sub(e, o));
-    }
-    f[0] = A::fma(keep, f[0], A::fma(-2.0, even.get(), orho));
-}
-
 // Component s of a pair of vectors.
 template <class C> __device__ __forceinline__ void node_part(const Two<C> (&v)[3], int s, C (&o)[3]) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) o[d] = s == 0 ? v[d].a : v[d].b;
-}
-
-// One species.
-template <class L> __device__ __forceinline__ void node_relax_one(float (&f)[L::Q], float rho, const float (&u)[3], float omega) {
-    node_relax<L>(OneF<L, float>{f}, rho, u, omega);
-}
-template <class L>
-__device__ __forceinline__ void node_relax_one(double (&f)[L::Q], double rho, const double (&u)[3], double omega) {
-    node_relax64<L, false>(f, rho, u, u, omega);
 }
 
 // Collision of both species of one node: common velocity shifted by tau_s g_s.
@@ -321,9 +275,9 @@ __device__ __forceinline__ void node_collide(C (&f)[2][L::Q], C rA, C rB, const 
     } else {
         C us[3];
         node_part<C>(u, 0, us);
-        node_relax_one<L>(f[0], rA, us, omega_A);
+        node_relax<L>(OneF<L, C>{f[0]}, rA, us, omega_A);
         node_part<C>(u, 1, us);
-        node_relax_one<L>(f[1], rB, us, omega_B);
+        node_relax<L>(OneF<L, C>{f[1]}, rB, us, omega_B);
     }
 }
 
@@ -389,9 +343,9 @@ __device__ __forceinline__ void node_collide_guo(C (&f)[2][L::Q], C rA, C rB, co
         C us[3], Fs[3];
         node_part<C>(u, 0, us);
         node_part<C>(F, 0, Fs);
-        node_relax64<L, true>(f[0], rA, us, Fs, omega_A);
+        node_relax_guo<L>(OneF<L, C>{f[0]}, rA, us, Fs, omega_A);
         node_part<C>(F, 1, Fs);
-        node_relax64<L, true>(f[1], rB, us, Fs, omega_B);
+        node_relax_guo<L>(OneF<L, C>{f[1]}, rB, us, Fs, omega_B);
     }
 }
 
