@@ -333,7 +333,8 @@ __device__ __forceinline__ void node_collide_guo(C (&f)[2][L::Q], C rA, C rB, co
     const C inv_den = A::rcp(A::fma(rA, omega_A, A::mul(rB, omega_B)));
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        F[d] = Ar2<C>::mul(rho, Two<C>{gA[d], gB[d]});
+        // rounded before c.F of the diagonal directions adds its components (Ar2: mul_split)
+        F[d] = Ar2<C>::mul_split(rho, Two<C>{gA[d], gB[d]});
         const Two<C> m = Ar2<C>::fma(both((C)0.5), F[d], j[d]);
         u[d] = both(A::mul(A::fma(m.a, omega_A, A::mul(m.b, omega_B)), inv_den));
     }
