@@ -43,6 +43,12 @@ struct Geometry {
     double dk[3];  // 2 pi / n of each axis
 };
 
+// Products and sums rounded as written, where several kernels form the same value.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
 // Wavenumbers of complex coefficient c (x the half axis, fastest): the full
 // ones (Laplacian) and the first-derivative ones (Nyquist of an even axis
 // zeroed), in the solver's precision T (FP32 arithmetic for the FP32 solver:
@@ -66,7 +72,7 @@ template <class T> __device__ __forceinline__ Wave<T> wave_at(const Geometry& g,
     wave_axis<T>(g, 1, iy, w.k[1], w.kd[1]);
     w.k[2] = w.kd[2] = (T)0;
     if (g.dim == 3) wave_axis<T>(g, 2, iz, w.k[2], w.kd[2]);
-    w.k2 = w.k[0] * w.k[0] + w.k[1] * w.k[1] + w.k[2] * w.k[2];
+    w.k2 = fma_rn(w.k[2], w.k[2], fma_rn(w.k[1], w.k[1], mul_rn(w.k[0], w.k[0])));
     return w;
 }
 template <class T> __device__ __forceinline__ Wave<T> wave_of(const Geometry& g, long long c) {
@@ -93,6 +99,8 @@ template <class C, class T> __device__ __forceinline__ C cscale(C a, T s) {
     r.y = s * a.y;
     return r;
 }
+// s a, rounded: a transform's first additions may not take the product up.
+__device__ __forceinline__ double2 cscale_rn(double2 a, double s) { return double2{mul_rn(s, a.x), mul_rn(s, a.y)}; }
 
 // 1. the inverse-transform inputs: phi^, i kd_a phi^, -k^2 phi^, u^_a (each / N)
 template <class T>
@@ -171,14 +179,18 @@ __device__ __forceinline__ void update_coeff(const Geometry& g, const Coeffs& c,
                                              int iz, C& p, C (&u)[D], C& s, C (&n)[D], const C& s_prev, const C (&n_prev)[D]) {
     const T Dc = (T)c.Dc, dt = (T)c.dt, nu = (T)c.nu;
     const T bi = (T)(c.Dc * (c.xi2 - c.dt * c.Dc / 2.0));
-    const T half = (T)0.5, three = (T)3;
-    const T k2 = w.k2, k4 = k2 * k2;
-    s.x -= bi * k4 * p.x;
-    s.y -= bi * k4 * p.y;
+    const T half = (T)0.5, one = (T)1, three = (T)3;
+    const T k2 = w.k2, k4 = mul_rn(k2, k2), bk = mul_rn(bi, k4);
+    s.x = fma_rn(-bk, p.x, s.x);
+    s.y = fma_rn(-bk, p.y, s.y);
     const C sp = first ? s : s_prev;
-    const T lam = Dc * ((T)2 * k2 + dt * Dc * half * k4);
-    const T am = (T)1 - dt * lam * half, inv_ap = (T)1 / ((T)1 + dt * lam * half);
-    p = C{(am * p.x + dt * (three * s.x - sp.x) * half) * inv_ap, (am * p.y + dt * (three * s.y - sp.y) * half) * inv_ap};
+    // (a x + dt (3 s - s') / 2) / b of one component, inv = 1 / b
+    auto advance = [&](T a, T x, T cur, T old, T inv) {
+        return mul_rn(fma_rn(a, x, mul_rn(mul_rn(dt, fma_rn(three, cur, -old)), half)), inv);
+    };
+    const T lam = mul_rn(Dc, fma_rn(mul_rn(mul_rn(dt, Dc), half), k4, mul_rn((T)2, k2)));
+    const T hl = mul_rn(mul_rn(dt, lam), half), am = one - hl, inv_ap = one / (one + hl);
+    p = C{advance(am, p.x, s.x, sp.x, inv_ap), advance(am, p.y, s.y, sp.y, inv_ap)};
     // Kolmogorov forcing A sin(2 pi y/ny) e_x: -i A N/2 at ky = +1, +i A N/2 at ky = -1 (kx = kz = 0)
     if (c.body_half_n != 0.0 && g.ny > 2 && ix == 0 && iz == 0) {
         if (iy == 1) n[0].y -= (T)c.body_half_n;
@@ -187,20 +199,19 @@ __device__ __forceinline__ void update_coeff(const Geometry& g, const Coeffs& c,
     T kd2 = 0, kre = 0, kim = 0;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        kd2 += w.kd[a] * w.kd[a];
-        kre += w.kd[a] * n[a].x;
-        kim += w.kd[a] * n[a].y;
+        kd2 = fma_rn(w.kd[a], w.kd[a], kd2);
+        kre = fma_rn(w.kd[a], n[a].x, kre);
+        kim = fma_rn(w.kd[a], n[a].y, kim);
     }
-    const T inv = kd2 > (T)0 ? (T)1 / kd2 : (T)0;
+    const T inv = kd2 > (T)0 ? one / kd2 : (T)0;
     const bool mean = k2 == (T)0;
-    const T vis = nu * k2;
-    const T bm = (T)1 - dt * vis * half, inv_bp = (T)1 / ((T)1 + dt * vis * half);
+    const T hv = mul_rn(mul_rn(dt, mul_rn(nu, k2)), half), bm = one - hv, inv_bp = one / (one + hv);
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        n[a] = mean ? C{(T)0, (T)0} : C{n[a].x - w.kd[a] * kre * inv, n[a].y - w.kd[a] * kim * inv};
+        n[a] = mean ? C{(T)0, (T)0}
+                    : C{fma_rn(-mul_rn(w.kd[a], kre), inv, n[a].x), fma_rn(-mul_rn(w.kd[a], kim), inv, n[a].y)};
         const C prev = first ? n[a] : n_prev[a];
-        u[a] = C{(bm * u[a].x + dt * (three * n[a].x - prev.x) * half) * inv_bp,
-                 (bm * u[a].y + dt * (three * n[a].y - prev.y) * half) * inv_bp};
+        u[a] = C{advance(bm, u[a].x, n[a].x, prev.x, inv_bp), advance(bm, u[a].y, n[a].y, prev.y, inv_bp)};
     }
 }
 
@@ -263,6 +274,9 @@ constexpr int kColThreads = 512;
 // derivative along this axis is still to be taken) are transformed and the state is
 // advanced.  INV: phi, its derivative along this axis, its second one and u go out.
 // in may be out: a block reads its own columns of every field before it writes.
+// Its arithmetic outside the transforms is rounded as written (mul_rn, fma_rn), so a
+// step gives the same bits whether it is the first of a call, in the middle or the
+// last: left to the compiler, the three kernels contracted different pairs.
 template <int D, bool FWD, bool INV>
 __global__ void __launch_bounds__(kColThreads)
     pfm_spectral_kernel(Geometry g, Coeffs c, pfm_fft::Plan plan, const double2* __restrict__ tw, int M,
@@ -293,8 +307,9 @@ __global__ void __launch_bounds__(kColThreads)
 #pragma unroll
         for (int q = 0; q < R0; ++q) {
             const Wave<T> w = D == 3 ? wave_at<T>(g, ix, iy3, col.row(q)) : wave_at<T>(g, ix, col.row(q), 0);
-            s[q].x -= (T)c.Dc * w.k2 * v[q].x;
-            s[q].y -= (T)c.Dc * w.k2 * v[q].y;
+            const T dk = mul_rn((T)c.Dc, w.k2);
+            s[q].x = fma_rn(-dk, v[q].x, s[q].x);
+            s[q].y = fma_rn(-dk, v[q].y, s[q].y);
         }
 #pragma unroll
         for (int a = 0; a < D; ++a) {
@@ -306,8 +321,8 @@ __global__ void __launch_bounds__(kColThreads)
             for (int q = 0; q < R0; ++q) {
                 T k, kd;
                 wave_axis<T>(g, D - 1, col.row(q), k, kd);
-                n[a][q].x += kd * v[q].y;
-                n[a][q].y -= kd * v[q].x;
+                n[a][q].x = fma_rn(kd, v[q].y, n[a][q].x);
+                n[a][q].y = fma_rn(-kd, v[q].x, n[a][q].y);
             }
         }
         load(st.phi, p);
@@ -352,26 +367,26 @@ __global__ void __launch_bounds__(kColThreads)
                 if (on) out[f * F + at(q)] = v[q];
         };
 #pragma unroll
-        for (int q = 0; q < R0; ++q) v[q] = p[q] = cscale(p[q], inv_n);
+        for (int q = 0; q < R0; ++q) v[q] = p[q] = cscale_rn(p[q], inv_n);
         send(0);
 #pragma unroll
         for (int q = 0; q < R0; ++q) {
             T k, kd;
             wave_axis<T>(g, D - 1, col.row(q), k, kd);
-            v[q] = cmul_i(p[q], kd);
+            v[q] = C{mul_rn(-kd, p[q].y), mul_rn(kd, p[q].x)};
         }
         send(1);
 #pragma unroll
         for (int q = 0; q < R0; ++q) {
             T k, kd;
             wave_axis<T>(g, D - 1, col.row(q), k, kd);
-            v[q] = cscale(p[q], -k * k);
+            v[q] = cscale_rn(p[q], -k * k);
         }
         send(2);
 #pragma unroll
         for (int a = 0; a < D; ++a) {
 #pragma unroll
-            for (int q = 0; q < R0; ++q) v[q] = cscale(n[a][q], inv_n);
+            for (int q = 0; q < R0; ++q) v[q] = cscale_rn(n[a][q], inv_n);
             send(3 + a);
         }
     }
