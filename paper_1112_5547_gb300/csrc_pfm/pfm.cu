@@ -20,6 +20,7 @@
 
 #include <cstdint>
 #include <cstring>
+#include <atomic>
 #include <new>
 
 #include "../../include/pfm.h"
@@ -659,6 +660,8 @@ __global__ void __launch_bounds__(kRowThreads, 2)
     }
 }
 
+constexpr size_t kFusedSmem = 200 * 1024;  // dynamic shared memory a fused kernel may use (bytes)
+
 // Shapes of the fused kernels.  They take FP64, even nx (at least 32: the x kernel's
 // fields then fit the room of the real ones) whose half, and ny and nz, are
 // 16 times factors 2, 3, 4, 5, up to the lengths whose lines fit shared memory;
@@ -682,7 +685,7 @@ inline int fused_columns(const pfm_fft::Plan& p, int nxh, long long lines) {
 Fused fused_shape(const Geometry& g, bool fp64) {
     Fused f;
     memset(&f, 0, sizeof(f));
-    const size_t smem = 200 * 1024;
+    const size_t smem = kFusedSmem;
     if (!fp64 || g.nx % 2 != 0 || g.nx < 32 || g.nx > 2048 || g.ny > 1024 || g.nz > 1024) return f;
     // small boxes: a block's chain of fourteen transforms is longer than the batched
     // ones' launches (32^3 164 against 118 us a step; 48 x 64 x 96 542 against 726)
@@ -861,11 +864,25 @@ template <class T> lbm_status step_typed(pfm_handle* h) {
     return LBM_OK;
 }
 
-template <class K> lbm_status launch_fused(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, void** args) {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return LBM_ERR_CUDA;
-    return cudaLaunchKernel((const void*)kern, grid, dim3(threads), args, smem, st) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+// The fused kernels may use kFusedSmem bytes of dynamic shared memory: asked for
+// once per kernel and device, never less, so that solvers of several sizes may be
+// stepped from several threads (the limit belongs to the kernel, not to a launch).
+template <auto Kern> cudaError_t fused_smem_once() {
+    constexpr int kMaxDevices = 64;
+    static std::atomic<int> done[kMaxDevices];  // zero-initialised: not yet set
+    int dev = 0;
+    const cudaError_t d = cudaGetDevice(&dev);
+    if (d != cudaSuccess) return d;
+    const bool known = dev >= 0 && dev < kMaxDevices;
+    if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem);
+    if (e == cudaSuccess && known) done[dev].store(1, std::memory_order_release);
+    return e;
+}
+
+template <auto Kern> lbm_status launch_fused(dim3 grid, int threads, size_t smem, cudaStream_t st, void** args) {
+    if (fused_smem_once<Kern>() != cudaSuccess) return LBM_ERR_CUDA;
+    return cudaLaunchKernel((const void*)Kern, grid, dim3(threads), args, smem, st) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
 // Fused steps: the spectral axis sends the state inwards, then per step y, x, y
@@ -884,8 +901,8 @@ template <int D> struct FusedRun {
         State st{at(h->L.phi_h), at(h->L.u_h), at(h->L.s_prev), at(h->L.n_prev)};
         const dim3 grid((unsigned)((g.nxh + M - 1) / M), D == 3 ? (unsigned)g.ny : 1u);
         void* args[] = {&h->g, &h->c, (void*)&p, &tw, &M, &first, &in, &out, &st};
-        return launch_fused(pfm_spectral_kernel<D, FWD, INV>, grid, p.n / R0 * M, pfm_fft::columns_smem(p.n, M), h->stream,
-                            args);
+        return launch_fused<pfm_spectral_kernel<D, FWD, INV>>(grid, p.n / R0 * M, pfm_fft::columns_smem(p.n, M), h->stream,
+                                                              args);
     }
     lbm_status y(bool inverse, C* in, C* out) const {
         const Geometry& g = h->g;
@@ -894,8 +911,9 @@ template <int D> struct FusedRun {
         C* tw = at(h->L.tw[1]);
         const dim3 grid((unsigned)((g.nxh + M - 1) / M), (unsigned)g.nz);
         void* args[] = {&h->g, (void*)&p, &tw, &M, &in, &out};
-        return launch_fused(inverse ? pfm_y_inverse_kernel : pfm_y_forward_kernel, grid, p.n / R0 * M,
-                            pfm_fft::columns_smem(p.n, M), h->stream, args);
+        const size_t smem = pfm_fft::columns_smem(p.n, M);
+        return inverse ? launch_fused<pfm_y_inverse_kernel>(grid, p.n / R0 * M, smem, h->stream, args)
+                       : launch_fused<pfm_y_forward_kernel>(grid, p.n / R0 * M, smem, h->stream, args);
     }
     lbm_status x(C* in, C* out) const {
         const Geometry& g = h->g;
@@ -904,7 +922,7 @@ template <int D> struct FusedRun {
         const long long rows = (long long)g.ny * g.nz;
         const dim3 grid((unsigned)((rows + R - 1) / R));
         void* args[] = {&h->g, &h->c, &h->fused.x, &tw, &R, &in, &out};
-        return launch_fused(pfm_x_kernel<D>, grid, kRowThreads, x_smem(g.nx, D, R), h->stream, args);
+        return launch_fused<pfm_x_kernel<D>>(grid, kRowThreads, x_smem(g.nx, D, R), h->stream, args);
     }
     lbm_status run(int nsteps) const {
         C* const cin = at(h->L.cin);
