@@ -662,10 +662,10 @@ __global__ void __launch_bounds__(kRowThreads, 2)
 
 constexpr size_t kFusedSmem = 200 * 1024;  // dynamic shared memory a fused kernel may use (bytes)
 
-// Shapes of the fused kernels.  They take FP64, even nx (at least 32: the x kernel's
-// fields then fit the room of the real ones) whose half, and ny and nz, are
-// 16 times factors 2, 3, 4, 5, up to the lengths whose lines fit shared memory;
-// other sizes go through cuFFT (ok = false).
+// Shapes of the fused kernels.  They take FP64, even nx whose half, and ny and nz, are
+// 16 times factors 2, 3, 4, 5, up to the lengths whose lines fit shared memory, and the
+// boxes that give the blocks of every axis enough SMs to run on (fused_pays); other
+// sizes go through cuFFT (ok = false).
 struct Fused {
     bool ok;
     pfm_fft::Plan x, y, z;
@@ -682,14 +682,29 @@ inline int fused_columns(const pfm_fft::Plan& p, int nxh, long long lines) {
     return M;
 }
 
+// Whether the fused kernels are faster than the batched transforms: a block's chain
+// of transforms is longer than the batched ones' launches, and its axis' blocks are
+// few where the box is small or narrow.  Measured (GB300, us a step, batched / fused):
+//   2D, 98304 nodes: 96 x 960 (just below) 218 / 183, 128 x 768 209 / 161; fewer: 128 x 512 127 / 130, 256 x 256 123 / 136,
+//       64 x 1024 133 / 160, 16 x 960 78 / 148
+//   2D, nx > 256 (more than 64 blocks of two columns): 400 x 288 248 / 223, 1024 x 288 545 / 489; narrower:
+//       1024 x 256 444 / 447, 384 x 256 191 / 189, 1024 x 128 321 / 376, 640 x 128 178 / 256
+//   2D, nx <= 1024: 512 x 1024 852 / 659; longer (the row kernel's first pass has 160 butterflies for its 256 threads
+//       at 1280, and one block an SM): 512 x 1280 993 / 1063, 1024 x 1280 2021 / 1795, 48 x 1440 150 / 232
+//   3D, 131072 nodes: 32 x 64 x 64 265 / 243; fewer: 32^3 118 / 164
+//   3D, nx >= 64: 512 x 32 x 64 1938 / 1672; narrower: 512 x 32 x 32 951 / 1181, 64 x 64 x 32 259 / 278
+//   3D, nz >= 32 (16 leave a block of the z kernel half a warp) unless rows are longer:
+//       16 x 96 x 96 361 / 352, 16 x 512 x 64 961 / 1011, 16 x 128 x 64 275 / 293
+inline bool fused_pays(const Geometry& g) {
+    if (g.dim == 2) return g.nreal >= 98304 && g.nx > 256 && g.nx <= 1024;
+    return g.nreal >= 131072 && g.nx >= 64 && (g.nz >= 32 || g.nx >= 96);
+}
+
 Fused fused_shape(const Geometry& g, bool fp64) {
     Fused f;
     memset(&f, 0, sizeof(f));
     const size_t smem = kFusedSmem;
-    if (!fp64 || g.nx % 2 != 0 || g.nx < 32 || g.nx > 2048 || g.ny > 1024 || g.nz > 1024) return f;
-    // small boxes: a block's chain of fourteen transforms is longer than the batched
-    // ones' launches (32^3 164 against 118 us a step; 48 x 64 x 96 542 against 726)
-    if (g.dim == 3 && g.nreal < 131072) return f;
+    if (!fp64 || g.nx % 2 != 0 || g.ny > 1024 || g.nz > 1024 || !fused_pays(g)) return f;
     if (!pfm_fft::make_plan(g.nx / 2, &f.x) || !pfm_fft::make_plan(g.ny, &f.y)) return f;
     if (g.dim == 3 && !pfm_fft::make_plan(g.nz, &f.z)) return f;
     f.My = fused_columns(f.y, g.nxh, g.nz);
@@ -927,7 +942,7 @@ template <int D> struct FusedRun {
     lbm_status run(int nsteps) const {
         C* const cin = at(h->L.cin);
         C* const cout = at(h->L.cout);
-        C* const mid = at(h->L.rphys);  // 10 spectral fields in the room of 11 real ones (nx >= 32)
+        C* const mid = at(h->L.rphys);  // 10 spectral fields in the room of 11 real ones (nx >= 64)
         lbm_status s = spectral<false, true>(cin, cin);
         for (int k = 0; k < nsteps && s == LBM_OK; ++k) {
             C* back = cout;
