@@ -188,10 +188,12 @@ cudaError_t init_typed(const Plan& p, const void* rA, const void* rB, const void
     const LatticeArgs<S> a = make_args<S>(p, nullptr, fout);
     if (zhi <= 0 || zhi > p.nz) zhi = p.nz;
     if (zlo < 0 || zlo >= zhi) return zlo == zhi ? cudaSuccess : cudaErrorInvalidValue;
-    const long long rows = (long long)(p.ny + 4) * (zhi - zlo);
-    const dim3 grid((unsigned)((p.nx + 2 * kInitLead + kInitThreads - 1) / kInitThreads), (unsigned)(rows < 32768 ? rows : 32768));
-    sc_init_kernel<L, S><<<grid, kInitThreads, 0, st>>>(a, static_cast<const C*>(rA), static_cast<const C*>(rB),
-                                                        static_cast<const C*>(u), zlo, zhi);
+    const InitRow row = init_row<S>(p.nx);
+    const long long cells = (long long)row.lanes * (p.ny + 4) * (zhi - zlo);
+    const int threads = cells < 65536 ? 64 : row.threads;  // few cells: every SM gets some
+    auto kern = u ? sc_init_kernel<L, S, true> : sc_init_kernel<L, S, false>;
+    kern<<<(unsigned)((cells + threads - 1) / threads), threads, 0, st>>>(
+        a, static_cast<const C*>(rA), static_cast<const C*>(rB), static_cast<const C*>(u), zlo, zhi);
     return cudaGetLastError();
 }
 

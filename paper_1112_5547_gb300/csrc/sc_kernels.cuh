@@ -590,75 +590,88 @@ __global__ void __launch_bounds__(NT) sc_diag_finish_kernel(const double* __rest
 // at node x holds f^eq_i(rho_s(x + c_i), u(x + c_i)), so pulling it at x + c_i
 // gives f_i(x + c_i, 0) = f^eq_i of that node.  The ghost columns and rows get
 // the values of their periodic images.
-// Threads run along the cells of a row (blockIdx.x) and the rows of planes
-// [zlo, zhi) are taken in turn (blockIdx.y): the periodic neighbours are three
-// indices per axis, formed once per cell.  The x images fill whole 32-byte
-// sectors and a warp's cells start on a cache line, as in store_node: rows begun
-// at the image column -2 left a partly written sector at either end of every
-// warp's stores, each of which reads HBM (512^3 FP32 8.2 ms, now 5.1; 4096^2 0.40,
-// now 0.29).
-constexpr int kInitThreads = 64, kInitLead = 32;
-template <class L, class S>
-__global__ void __launch_bounds__(kInitThreads)
+// One thread per cell, row after row.  Wide rows hold whole 32-byte sectors (the x images
+// fill one on either side, as in store_node), and their lanes begin on one, so that no warp's
+// stores leave a partly written sector, each of which reads HBM; 16-bit rows begin on a
+// cache line.  Narrow rows, where the images would be a good part of the work, take the
+// two images that a step reads.  Whether the fluid moves is a template argument: a branch
+// around the velocity's loads in each of the Q directions serialises them.  Measured
+// (GB300, us at rest / moving; rows walked by blocks of 64 lanes, with that branch, and
+// now): FP32 512^3 5214 / 9294 -> 3407 / 6175, 128^3 77 / 124 -> 59 / 119; FP64 160^3
+// 1261 / 3120 -> 627 / 2337, 171 x 217 x 4 529 / 1289 -> 102 / 172; bf16 rest-offset 256^3
+// 535 / 901 -> 453 / 697.
+struct InitRow {
+    int images;   // cells x in [-images, nx + images) are written
+    int lead;     // lane 0 is the cell x = -lead
+    int lanes;    // of a row
+    int threads;  // of a block
+};
+template <class S> __host__ __device__ __forceinline__ InitRow init_row(int nx) {
+    constexpr int kSector = 32 / (int)sizeof(S) > 2 ? 32 / (int)sizeof(S) : 2;
+    // rows of less than 12 sectors (FP32 185 x 158 x 78: 153 us with whole sectors, 145 without)
+    if (nx < 12 * kSector) return InitRow{2, 2, nx + 4, Codec<S>::kRest ? 64 : 256};
+    if (sizeof(S) == 2) return InitRow{kSector, 32, (nx + 32 + kSector + 31) / 32 * 32, 256};
+    return InitRow{kSector, kSector, (nx + 2 * kSector + kSector - 1) / kSector * kSector, 64};
+}
+template <class L, class S, bool MOVING>
+__global__ void __launch_bounds__(256)
     sc_init_kernel(const LatticeArgs<S> a, const typename Codec<S>::C* __restrict__ rhoA,
                    const typename Codec<S>::C* __restrict__ rhoB, const typename Codec<S>::C* __restrict__ u, int zlo,
                    int zhi) {
     using C = typename Codec<S>::C;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    constexpr int kSector = 32 / (int)sizeof(S) > 2 ? 32 / (int)sizeof(S) : 2;
-    const int GX = nx >= kSector ? kSector : 2;
-    const int ey = ny + 4;  // cells x in [-GX, nx + GX), y in [-2, ny + 2)
-    const int cx = (int)(blockIdx.x * kInitThreads + threadIdx.x) - kInitLead;
-    if (cx < -GX || cx >= nx + GX) return;
-    const int x = ((cx % nx) + nx) % nx;
-    const int xs[3] = {wrap_dec(x, nx), x, wrap_inc(x, nx)};
+    const InitRow rw = init_row<S>(nx);
+    const int ey = ny + 4;  // cells y in [-2, ny + 2)
+    const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    auto quotient = [](long long v, int d) { return v <= 0xffffffffLL ? (long long)((unsigned)v / (unsigned)d) : v / d; };
+    const long long row = quotient(k, rw.lanes), plane = quotient(row, ey);
+    const int cx = (int)(k - row * rw.lanes) - rw.lead;
+    const int cy = (int)(row - plane * ey) - 2;
     // the cells of planes [zlo, zhi); they read the fields of planes zlo - 1 .. zhi (periodic)
-    const long long rows = (long long)ey * (zhi - zlo);
-    for (long long row = blockIdx.y; row < rows; row += gridDim.y) {
-        const int cy = (int)(row % ey) - 2;
-        const int z = zlo + (int)(row / ey);
-        const size_t n = cell(a, cx, cy, z);
-        const int y = ((cy % ny) + ny) % ny;
-        const int ys[3] = {wrap_dec(y, ny), y, wrap_inc(y, ny)};
-        const int zs[3] = {L::D == 3 ? wrap_dec(z, nz) : 0, L::D == 3 ? z : 0, L::D == 3 ? wrap_inc(z, nz) : 0};
-        C fr[2][L::Q];  // rest-offset storage: the cell's values, stored together
+    if (cx < -rw.images || cx >= nx + rw.images || plane >= zhi - zlo) return;
+    const int z = zlo + (int)plane;
+    const size_t n = cell(a, cx, cy, z);
+    const int x = ((cx % nx) + nx) % nx, y = ((cy % ny) + ny) % ny;
+    const int xs[3] = {wrap_dec(x, nx), x, wrap_inc(x, nx)};
+    const int ys[3] = {wrap_dec(y, ny), y, wrap_inc(y, ny)};
+    const int zs[3] = {L::D == 3 ? wrap_dec(z, nz) : 0, L::D == 3 ? z : 0, L::D == 3 ? wrap_inc(z, nz) : 0};
+    C fr[2][L::Q];  // rest-offset storage: the cell's values, stored together
 #pragma unroll
-        for (int i = 0; i < L::Q; ++i) {
-            const size_t m = (size_t)xs[L::c(i, 0) + 1] +
-                             (size_t)nx * ((size_t)ys[L::c(i, 1) + 1] + (size_t)ny * zs[L::c(i, 2) + 1]);
-            C shape = (C)1;
-            if (u) {
-                C uv[3] = {0, 0, 0};
-                for (int d = 0; d < L::D; ++d) uv[d] = u[(size_t)d * (size_t)a.N + m];
-                C uu = uv[0] * uv[0] + uv[1] * uv[1] + uv[2] * uv[2];
-                C cu = (C)0;
-                for (int d = 0; d < L::D; ++d) cu += (C)L::c(i, d) * uv[d];
-                shape = (C)1 - (C)1.5 * uu + cu * ((C)3 + (C)4.5 * cu);
-            }
+    for (int i = 0; i < L::Q; ++i) {
+        const size_t m = (size_t)xs[L::c(i, 0) + 1] +
+                         (size_t)nx * ((size_t)ys[L::c(i, 1) + 1] + (size_t)ny * zs[L::c(i, 2) + 1]);
+        C shape = (C)1;
+        if (MOVING) {
+            C uv[3] = {0, 0, 0};
+            for (int d = 0; d < L::D; ++d) uv[d] = u[(size_t)d * (size_t)a.N + m];
+            C uu = uv[0] * uv[0] + uv[1] * uv[1] + uv[2] * uv[2];
+            C cu = (C)0;
+            for (int d = 0; d < L::D; ++d) cu += (C)L::c(i, d) * uv[d];
+            shape = (C)1 - (C)1.5 * uu + cu * ((C)3 + (C)4.5 * cu);
+        }
 #pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                // SC: species densities; FE: f from rho = rho_A + rho_B, g from phi = rho_A - rho_B
-                const C rho = a.model == kModelFE ? (s == 0 ? rhoA[m] + rhoB[m] : rhoA[m] - rhoB[m])
-                                                  : (s == 0 ? rhoA[m] : rhoB[m]);
-                const C f = (C)L::w(i) * rho * shape;
-                if constexpr (Codec<S>::kRest) {
-                    fr[s][i] = f;
-                } else {
-                    const C off = Codec<S>::kOffset ? (C)__fmul_rn((float)L::w(i), (float)(s == 0 ? a.ref_A : a.ref_B)) : (C)0;
-                    Codec<S>::store(a.fout + (size_t)(s * L::Q + i) * (size_t)a.Np + n, f, off);
-                }
+        for (int s = 0; s < 2; ++s) {
+            // SC: species densities; FE: f from rho = rho_A + rho_B, g from phi = rho_A - rho_B
+            const C rho = a.model == kModelFE ? (s == 0 ? rhoA[m] + rhoB[m] : rhoA[m] - rhoB[m])
+                                              : (s == 0 ? rhoA[m] : rhoB[m]);
+            const C f = (C)L::w(i) * rho * shape;
+            if constexpr (Codec<S>::kRest) {
+                fr[s][i] = f;
+            } else {
+                const C off = Codec<S>::kOffset ? (C)__fmul_rn((float)L::w(i), (float)(s == 0 ? a.ref_A : a.ref_B)) : (C)0;
+                Codec<S>::store(a.fout + (size_t)(s * L::Q + i) * (size_t)a.Np + n, f, off);
             }
         }
-        if constexpr (Codec<S>::kRest) {
-            // rest-offset bases: the sums of the cell's stored values, in a fixed order
-            float2 r = make_float2(fr[0][0], fr[1][0]);
+    }
+    if constexpr (Codec<S>::kRest) {
+        // rest-offset bases: the sums of the cell's stored values, in a fixed order
+        float2 r = make_float2(fr[0][0], fr[1][0]);
 #pragma unroll
-            for (int i = 1; i < L::Q; ++i) {
-                r.x = __fadd_rn(r.x, fr[0][i]);
-                r.y = __fadd_rn(r.y, fr[1][i]);
-            }
-            store_cell<L, S>(a, n, fr, r);
+        for (int i = 1; i < L::Q; ++i) {
+            r.x = __fadd_rn(r.x, fr[0][i]);
+            r.y = __fadd_rn(r.y, fr[1][i]);
         }
+        store_cell<L, S>(a, n, fr, r);
     }
 }
 
