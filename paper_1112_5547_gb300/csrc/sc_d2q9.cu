@@ -52,21 +52,34 @@ bool resident_allowed() {
 
 int resident_ctas(const Plan& p) { return p.ny / 2 < kResidentCtas ? p.ny / 2 : kResidentCtas; }
 
+// Threads of a CTA: a row of warps along x, as many rows as fit (no more than the band and its halo).
+dim3 resident_block(const Plan& p, int ctas) {
+    const int bx = (p.nx + 31) / 32 * 32, rows = d2_resident_rows(p.ny, ctas) + 2;
+    const int by = kResidentThreads / bx;
+    return dim3(bx, by < rows ? by : rows);
+}
+
+// Passes of a CTA over its band's rows in a step, at most.  One pass costs about 1.5 us, so
+// tall narrow lattices, a warp per row, are better off on all SMs: us for 3 / 5 / 100
+// steps, 400 x 30 (two passes) 13 / 18 / 249 and 9 / 15 / 271 on all SMs, 300 x 40 (three) 15 / 21 /
+// 325 and 9 / 15 / 295, 1000 x 8 (five) 23 / 32 / 451 and 11 / 18 / 354 (one launch a step
+// before chained launches: 19 / 31 / 615).
+constexpr int kResidentPasses = 3;
+
 }  // namespace
 
 bool d2q9_resident_fits(const Plan& p) {
     const int ctas = resident_ctas(p);
-    return p.lattice == 0 && p.precision == 1 && p.nx <= kResidentThreads && ctas >= 1 &&
-           p.N <= kResidentNodes && d2_resident_smem(p.nx, p.ny, ctas) <= kSmemPerCta && resident_allowed();
+    if (p.lattice != 0 || p.precision != 1 || p.nx > kResidentThreads || ctas < 1 || p.N > kResidentNodes) return false;
+    const int by = (int)resident_block(p, ctas).y;
+    return (d2_resident_rows(p.ny, ctas) + 2 + by - 1) / by <= kResidentPasses &&
+           d2_resident_smem(p.nx, p.ny, ctas) <= kSmemPerCta && resident_allowed();
 }
 
 cudaError_t d2q9_resident(const Plan& p, const void* fin, void* fout, int nsteps, cudaStream_t st) {
-    const int ctas = resident_ctas(p), bx = (p.nx + 31) / 32 * 32;
-    int by = kResidentThreads / bx;
-    const int rows = d2_resident_rows(p.ny, ctas) + 2;
-    if (by > rows) by = rows;
-    return launch_chained(sc_d2_resident_kernel<kResidentThreads>, dim3((unsigned)ctas), dim3(bx, by), d2_resident_smem(p.nx, p.ny, ctas),
-                          st, ctas, 1, make_args<float>(p, fin, fout), nsteps);
+    const int ctas = resident_ctas(p);
+    return launch_chained(sc_d2_resident_kernel<kResidentThreads>, dim3((unsigned)ctas), resident_block(p, ctas),
+                          d2_resident_smem(p.nx, p.ny, ctas), st, ctas, 1, make_args<float>(p, fin, fout), nsteps);
 }
 
 cudaError_t d2q9_init(const Plan& p, const void* rA, const void* rB, const void* u, void* fout, cudaStream_t st,
