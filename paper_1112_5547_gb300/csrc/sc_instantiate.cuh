@@ -20,7 +20,7 @@ cudaError_t step_tiled(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) 
     // 0.67 ms a step at 4096^2; two (128 registers) in FP64.
     constexpr int kMin = L::D == 2 ? (sizeof(C) == 8 ? 2 : 3) * (TX * TY <= 128 ? 2 : 1) / (TX * TY > 256 ? 2 : 1)
                          : sizeof(C) == 8 ? 1 : (TX * TY <= 128 ? 4 : (TX * TY <= 256 ? 2 : 1));
-    return launch_chained(sc_fused_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a);
+    return launch_register_kernel(p, sc_fused_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), st, a);
 }
 
 // Tile 3 in FP64 (D3Q19): 32x4 or 16x8 columns, whichever leaves fewer lanes
@@ -32,14 +32,14 @@ template <class L> cudaError_t step_f64_tile3(const Plan& p, const LatticeArgs<d
     if (tx == 32) return step_tiled<L, double, 32, 4>(p, a, st);
     const dim3 grid((unsigned)((p.nx + tx - 1) / tx), (unsigned)((p.ny + ty - 1) / ty),
                     (unsigned)((p.nz + p.step_zchunk - 1) / p.step_zchunk));
-    return launch_chained(sc_fused_kernel<L, double, 16, 8, 1>, grid, dim3(tx, ty), 0, st, 1, 1, a);
+    return launch_register_kernel(p, sc_fused_kernel<L, double, 16, 8, 1>, grid, dim3(tx, ty), st, a);
 }
 
 template <class L, class S, int TX, int TY, int MINB>
 cudaError_t step_reload(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) {
     using C = typename Codec<S>::C;
     constexpr int kMin = sizeof(C) == 8 ? (MINB > 2 ? MINB / 2 : 1) : MINB;
-    return launch_chained(sc_step_reload_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a);
+    return launch_register_kernel(p, sc_step_reload_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), st, a);
 }
 
 template <class L, class S, int TX, int TY, int ST, int FORCING = kForcingShift, int MINB = 1> struct TmaLaunch {
@@ -76,7 +76,7 @@ template <class S, int TX, int TY, int MINB> struct RegPipeLaunch<D3Q19, S, TX, 
         if constexpr (sizeof(S) == 8) {
             return cudaErrorInvalidValue;  // three planes of doubles do not fit in registers
         } else {
-            return launch_chained(sc_step_regpipe_kernel<S, TX, TY, MINB>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a);
+            return launch_register_kernel(p, sc_step_regpipe_kernel<S, TX, TY, MINB>, step_grid(p), dim3(TX, TY), st, a);
         }
     }
 };

@@ -148,26 +148,52 @@ inline bool tile_fits(int tile, const Plan& p) {
 // ended.  Steps come out 2 - 3 us shorter (us a step without and with: D2Q9
 // 64^2 6.2 / 2.7, 256^2 6.2 / 3.8; D3Q19 FP32 32^3 10.3 / 7.4, 64^3 30.9 / 28.7).
 template <class... KA, class... A>
-cudaError_t launch_chained(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cx, int cy,
-                           const A&... args) {
+cudaError_t launch_step_kernel(bool chained, void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                               int cx, int cy, const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 0;
+    if (chained) {
+        cudaLaunchAttribute& a = attr[cfg.numAttrs++];
+        a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        a.val.programmaticStreamSerializationAllowed = 1;
+    }
     if (cx > 1 || cy > 1) {
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = cx;
-        attr[1].val.clusterDim.y = cy;
-        attr[1].val.clusterDim.z = 1;
-        cfg.numAttrs = 2;
+        cudaLaunchAttribute& a = attr[cfg.numAttrs++];
+        a.id = cudaLaunchAttributeClusterDimension;
+        a.val.clusterDim.x = cx;
+        a.val.clusterDim.y = cy;
+        a.val.clusterDim.z = 1;
     }
     return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <class... KA, class... A>
+cudaError_t launch_chained(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cx, int cy,
+                           const A&... args) {
+    return launch_step_kernel(true, kern, grid, block, smem, st, cx, cy, args...);
+}
+
+// Whether the register kernels (several CTAs per SM) of a D3Q19 lattice are chained.  The next
+// step's CTAs are placed while this step's hold their slots, on the SMs that hold
+// fewest, and stay there: where the grid leaves slots free but is larger than the
+// SMs, some SMs then get two or three of them and others none.  Steps of some
+// microseconds gain more from the early launch; the others lose (GB300, us a step,
+// chained / not): FP64 56^3, 168 CTAs 325 / 208; FP64 tile 11 96^3 1006 / 700; FP32
+// tiles 13, 15 and 3 at 96^3 136 / 107, 122 / 91, 96 / 87; but FP32 30^3 - 48^3 10 - 20 % gained.
+// A grid of at most one CTA per SM stays even (FP64 16^3 - 32^3 2 - 8 % gained), and so do
+// the kernels with one CTA per SM and the small CTAs of D2Q9.
+inline bool chain_pays(const Plan& p, dim3 grid) {
+    if (p.lattice == 0 || (long long)grid.x * grid.y * grid.z <= p.sm_count) return true;
+    return p.N <= (p.precision == 0 || kTiles[p.step_tile].kind == 3 ? 32768 : 131072);
+}
+template <class... KA, class... A>
+cudaError_t launch_register_kernel(const Plan& p, void (*kern)(KA...), dim3 grid, dim3 block, cudaStream_t st, const A&... args) {
+    return launch_step_kernel(chain_pays(p, grid), kern, grid, block, 0, st, 1, 1, args...);
 }
 
 struct MomentsOut {
