@@ -39,6 +39,8 @@ template <class L, class S, int TX, int TY, int MINB>
 cudaError_t step_reload(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) {
     using C = typename Codec<S>::C;
     constexpr int kMin = sizeof(C) == 8 ? (MINB > 2 ? MINB / 2 : 1) : MINB;
+    if constexpr (reload_nc<L, S, TX, TY, kMin>())
+        return launch_step_kernel(false, sc_step_reload_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), 0, st, 1, 1, a);
     return launch_register_kernel(p, sc_step_reload_kernel<L, S, TX, TY, kMin>, step_grid(p), dim3(TX, TY), st, a);
 }
 

@@ -30,7 +30,8 @@
 namespace lbmsc {
 
 // Pulled populations of node (x, y, z): f_is = f*_is(x - c_i).
-template <class L, class S>
+// NC: through the non-coherent path (kernels that are not chained only).
+template <class L, class S, bool NC = false>
 __device__ __forceinline__ void pull_node(const LatticeArgs<S>& a, int x, int y, int z,
                                           typename Codec<S>::C (&f)[2][L::Q]) {
     using C = typename Codec<S>::C;
@@ -51,7 +52,11 @@ __device__ __forceinline__ void pull_node(const LatticeArgs<S>& a, int x, int y,
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
                 const C off = Codec<S>::kOffset ? (C)__fmul_rn((float)L::w(i), (float)(s == 0 ? a.ref_A : a.ref_B)) : (C)0;
-                f[s][i] = Codec<S>::load(a.fin + (size_t)(s * L::Q + i) * (size_t)a.Np + node, off);
+                const S* const src = a.fin + (size_t)(s * L::Q + i) * (size_t)a.Np + node;
+                if constexpr (NC)
+                    f[s][i] = Codec<S>::decode(__ldg(src), off);
+                else
+                    f[s][i] = Codec<S>::load(src, off);
             }
         }
     }
@@ -501,6 +506,14 @@ __global__ void __launch_bounds__(TX* TY, MINB)
 // they are normally still in L1.  Holding only one plane of pulls lets more
 // CTAs share an SM (more loads in flight), and the four-slot density ring
 // needs one __syncthreads per plane.  Arithmetic and order as sc_fused_kernel.
+// Reference-offset 16-bit storage on tile 14 (D3Q19, 128 registers a thread): the pulls go
+// through the non-coherent path, which lets the compiler move them across the
+// plane's barrier (48^3, 16 planes a chunk: 70 us a step with plain loads, 55 so); such
+// a kernel is not chained (sc_common.cuh).  In the other storages and tiles plain loads
+// are as fast or faster (rest-offset by up to 14 %).
+template <class L, class S, int TX, int TY, int MINB> constexpr bool reload_nc() {
+    return L::D == 3 && Codec<S>::kOffset && TX * TY * MINB <= 512;
+}
 template <class L, class S, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const LatticeArgs<S> a) {
     using C = typename Codec<S>::C;
@@ -509,9 +522,12 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
     constexpr int NPL = L::D == 3 ? 4 : 1;
     constexpr int H = 2 * FX + 2 * TY;
     static_assert(H <= TX * TY, "halo ring must fit in the CTA");
+    constexpr bool NC = reload_nc<L, S, TX, TY, MINB>();
     __shared__ Two<C> ring[NPL][FY][FX];
-    chain_wait();
-    chain_next();
+    if (!NC) {
+        chain_wait();
+        chain_next();
+    }
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -526,16 +542,25 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
 
     auto density_plane = [&](int slot, int z) {
         C f[2][Q];
-        pull_node<L, S>(a, gx, gy, z, f);
+        pull_node<L, S, NC>(a, gx, gy, z, f);
         ring[slot][ty + 1][tx + 1] = node_densities<L, C>(f);
         if (halo) {
-            pull_node<L, S>(a, hgx, hgy, z, f);
+            pull_node<L, S, NC>(a, hgx, hgy, z, f);
             ring[slot][hfy][hfx] = node_densities<L, C>(f);
         }
     };
-    auto collide = [&](int sm, int sc, int sp, int z) {
+    // (kept == nullptr: pull here)
+    auto collide = [&](C (*kept)[2][Q], int sm, int sc, int sp, int z) {
         C f[2][Q];
-        pull_node<L, S>(a, gx, gy, z, f);
+        if (kept) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                f[0][i] = (*kept)[0][i];
+                f[1][i] = (*kept)[1][i];
+            }
+        } else {
+            pull_node<L, S, NC>(a, gx, gy, z, f);
+        }
         const Two<C> r = ring[sc][ty + 1][tx + 1];
         const C rA = r.a, rB = r.b;
         auto nbr = [&](int i) -> Two<C> {
@@ -547,9 +572,18 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
     };
 
     if (L::D == 2) {
-        density_plane(0, 0);
+        // one plane: its pulls stay in registers (pulled again, 2000 x 2100 bf16
+        // rest-offset on tile 11 takes 160 us a step instead of 106)
+        C f[2][Q];
+        pull_node<L, S>(a, gx, gy, 0, f);
+        ring[0][ty + 1][tx + 1] = node_densities<L, C>(f);
+        if (halo) {
+            C h[2][Q];
+            pull_node<L, S>(a, hgx, hgy, 0, h);
+            ring[0][hfy][hfx] = node_densities<L, C>(h);
+        }
         __syncthreads();
-        collide(0, 0, 0, 0);
+        collide(&f, 0, 0, 0, 0);
         return;
     }
     const int z0 = blockIdx.z * a.zchunk;
@@ -562,7 +596,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) sc_step_reload_kernel(const Latt
         const int k = z - z0 + 1;
         density_plane((k + 1) & 3, z + 1 == nz ? 0 : z + 1);
         __syncthreads();
-        collide((k - 1) & 3, k & 3, (k + 1) & 3, z);
+        collide(nullptr, (k - 1) & 3, k & 3, (k + 1) & 3, z);
     }
 }
 
