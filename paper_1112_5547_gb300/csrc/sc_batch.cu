@@ -78,8 +78,11 @@ cudaError_t launch_batch_tma(const void* lats, const BatchItem* items, int nitem
     long long grid = grid_mode ? nitems : sm_count;
     if (grid > nitems) grid = nitems;
     if (grid < 1) return cudaSuccess;
-    return launch_chained(kern, dim3((unsigned)grid), dim3(TX, TY), T::smem_bytes, st, 1, 1,
-                          static_cast<const BatchTmaLattice*>(lats), items, nitems, parity, grid_mode ? nullptr : ctr);
+    // 32x12 tiles: CTAs started ahead of the others on the SMs that come free drift from
+    // their neighbours' halo rows (100 x 70 x 60 x 8 488 us a step chained, 460 not; 64^3 x 20 550 / 536)
+    const bool chained = TX * TY <= 256 || grid <= sm_count;
+    return launch_step_kernel(chained, kern, dim3((unsigned)grid), dim3(TX, TY), T::smem_bytes, st, 1, 1,
+                              static_cast<const BatchTmaLattice*>(lats), items, nitems, parity, grid_mode ? nullptr : ctr);
 }
 
 template <int WX, int WY, int NX, int NY, int S>

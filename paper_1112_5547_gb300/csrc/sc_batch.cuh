@@ -218,8 +218,12 @@ __global__ void __launch_bounds__(TX* TY, 1)
                 }
             }
         };
-        const int n = tma_item<TX, TY, S>(&l->map[parity], nullptr, a, w.x0, w.y0, w.z0, qbase, sm, l->err,
-                                          preissued, &nxt, hook, true);
+        // 384 threads have 168 registers each: with the next item's state in them the
+        // packed relaxation spills (168 bytes; 64^3 x 20 on this tile 652 us a step, one species
+        // after the other 552)
+        constexpr bool kPack = TX * TY <= 256;
+        const int n = tma_item<TX, TY, S, float, decltype(hook), kForcingShift, kPack>(
+            &l->map[parity], nullptr, a, w.x0, w.y0, w.z0, qbase, sm, l->err, preissued, &nxt, hook, true);
         if (n < 0) break;  // a lost wait: the lattice's error word is raised
         qbase += (unsigned)n;
         // the next item's first planes went out with this one (the elected

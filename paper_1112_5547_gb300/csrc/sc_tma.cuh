@@ -271,7 +271,9 @@ struct TmaNoHook {
 // raised, and the copies still in flight have been waited for, again with a
 // bound).  The caller must synchronise the CTA between two items.
 // alternate: odd chunks march downwards (tma_march_down; batch kernels).
-template <int TX, int TY, int S, class St = float, class Hook = TmaNoHook, int FORCING = kForcingShift>
+// PACK: both species relax together (node_collide).
+template <int TX, int TY, int S, class St = float, class Hook = TmaNoHook, int FORCING = kForcingShift,
+          bool PACK = std::is_same<St, float>::value>
 __device__ __forceinline__ int tma_item(const CUtensorMap* pmap, const CUtensorMap* rmap, const LatticeArgs<St>& a,
                                         int x0, int y0, int z0, unsigned qbase, const TmaSmem<TX, TY, S, St>& sm,
                                         int* __restrict__ err, bool preissued = false, const TmaNext* nxt = nullptr,
@@ -388,7 +390,7 @@ __device__ __forceinline__ int tma_item(const CUtensorMap* pmap, const CUtensorM
             if constexpr (FORCING == kForcingGuo)
                 node_collide_guo<L, C>(X, rA, rB, gA, gB, a.omega_A, a.omega_B);
             else
-                node_collide<L, C, std::is_same<St, float>::value>(X, rA, rB, gA, gB, a.omega_A, a.omega_B, a.tau_A, a.tau_B);
+                node_collide<L, C, PACK>(X, rA, rB, gA, gB, a.omega_A, a.omega_B, a.tau_A, a.tau_B);
         }
         if (owner) store_node<L, St>(a, gx, gy, zof(q), X, rA, rB);
     };
