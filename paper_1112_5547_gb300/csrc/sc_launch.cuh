@@ -209,7 +209,10 @@ struct MomentsOut {
 // Grid of the moments kernel over `planes` planes: items of one tile and one z
 // chunk, the chunk chosen for the shortest time on 152 SMs with three CTAs each
 // (a chunk of zc planes pulls two more), and the CTAs of a diagnostics launch,
-// which take the items in turn and leave one record of partial sums each.
+// which take the items in turn and leave one record of partial sums each.  In FP64
+// an SM's CTAs share its FP64 units, so it counts as one (three a SM gave shorter
+// chunks: fields of 5 x 93 x 270 96 us and of 48^3 84, now 86 and 72).  The shape, and with it
+// the records' place in a workspace, does not depend on the device.
 struct MomentsShape {
     int tiles_x, tiles_y, zchunk, items, ctas;
 };
@@ -219,11 +222,11 @@ inline MomentsShape moments_shape(const Plan& p, int planes) {
     m.tiles_x = (p.nx + kTX - 1) / kTX;
     m.tiles_y = (p.ny + kTY - 1) / kTY;
     m.zchunk = 1;
-    const long long xy = (long long)m.tiles_x * m.tiles_y;
+    const long long xy = (long long)m.tiles_x * m.tiles_y, slots = p.precision == 0 ? 152 : 3 * 152;
     long long best = -1;
     if (p.lattice == 1)
         for (int zc = 1; zc <= planes && zc <= 32; ++zc) {
-            const long long n = xy * ((planes + zc - 1) / zc), cost = ((n + 455) / 456) * (zc + 2);
+            const long long n = xy * ((planes + zc - 1) / zc), cost = ((n + slots - 1) / slots) * (zc + 2);
             if (best < 0 || cost < best) {
                 best = cost;
                 m.zchunk = zc;
