@@ -196,7 +196,8 @@ typedef struct lbm_sc_handle lbm_sc_handle;
  * overlaps the other's work).  With LBM_FORCING_GUO or
  * LBM_MODEL_FE the accepted tiles are those of the register and low-register
  * kernels (0-4, 11-14) and the TMA tile 34.  zchunk is the number
- * of z planes each CTA marches over per work item (D3Q19 only; 0 = automatic).
+ * of z planes each CTA marches over per work item (D3Q19 only; 0 = automatic: the
+ * chunk that a lattice without tuning takes on that tile).
  * The shape changes only speed: every shape computes bit-identical results. */
 typedef struct {
     int32_t tile;
@@ -217,7 +218,8 @@ LBM_SC_API lbm_status lbm_sc_create(const lbm_sc_params* params, void* d_workspa
 
 /* Set / read the launch shape of the step kernel (see lbm_sc_tuning).
  * LBM_ERR_INVALID_ARG for an unknown tile, a tile the lattice and precision
- * do not support, or a negative zchunk. */
+ * do not support, a negative zchunk, or more than 65535 tile rows or z chunks
+ * (no launch takes them). */
 LBM_SC_API lbm_status lbm_sc_set_tuning(lbm_sc_handle* h, const lbm_sc_tuning* tuning);
 LBM_SC_API lbm_status lbm_sc_get_tuning(const lbm_sc_handle* h, lbm_sc_tuning* tuning);
 

@@ -73,21 +73,6 @@ bool valid(const lbm_sc_params* p) {
     return true;
 }
 
-// Planes per CTA along z: enough work items to fill the 152 SMs several times
-// over, at least min_planes planes per chunk so the two extra density planes
-// of each chunk stay cheap.
-int pick_zchunk(const lbm_sc_params* p, int tx = lbmsc::kTX, int ty = lbmsc::kTY, long long target = 152LL * 2 * 8,
-                int min_planes = 16) {
-    if (p->lattice == LBM_D2Q9) return 1;
-    const long long tiles = (long long)((p->nx + tx - 1) / tx) * ((p->ny + ty - 1) / ty);
-    long long chunks = (target + tiles - 1) / tiles;
-    long long max_chunks = p->nz / min_planes;
-    if (max_chunks < 1) max_chunks = 1;
-    if (chunks > max_chunks) chunks = max_chunks;
-    if (chunks < 1) chunks = 1;
-    return (int)((p->nz + chunks - 1) / chunks);
-}
-
 Plan make_plan(const lbm_sc_params* p) {
     Plan pl{};
     pl.lattice = p->lattice;
@@ -201,10 +186,14 @@ lbm_status lbm_sc_create(const lbm_sc_params* p, void* d_workspace, size_t works
 lbm_status lbm_sc_set_tuning(lbm_sc_handle* h, const lbm_sc_tuning* t) {
     if (!h || !t || t->zchunk < 0) return LBM_ERR_INVALID_ARG;
     if (!lbmsc::tile_fits(t->tile, h->plan)) return LBM_ERR_INVALID_ARG;
-    const lbmsc::TileShape ts = lbmsc::kTiles[t->tile];
+    int zc = 1;
+    if (h->params.lattice == LBM_D3Q19) {
+        // 0: the chunk an untuned lattice takes on this tile
+        zc = t->zchunk != 0 ? t->zchunk : lbmsc::best_zchunk(h->plan, t->tile);
+        if (zc > h->params.nz) zc = h->params.nz;
+    }
+    if (!lbmsc::shape_fits_grid(t->tile, zc, h->plan)) return LBM_ERR_INVALID_ARG;
     h->plan.step_tile = t->tile;
-    int zc = t->zchunk != 0 ? t->zchunk : pick_zchunk(&h->params, ts.tx, ts.ty);
-    if (h->params.lattice == LBM_D2Q9 || zc > h->params.nz) zc = h->params.lattice == LBM_D2Q9 ? 1 : h->params.nz;
     h->plan.step_zchunk = zc;
     return LBM_OK;
 }

@@ -64,8 +64,13 @@ inline StepModel step_model(const Plan& p, int tile) {
         case 38: return {1, 1.2, 0.78, 0.8};
         case 15:
         case 17: return {3, 2.0, l2 ? 0.85 : 1.5, 0.8};
-        default: return p.precision == 1 ? StepModel{4, 2.0, l2 ? 0.96 : 1.75, 0.8} : StepModel{4, 2.0, l2 ? 1.3 : 1.8, 0.8};
+        default: break;
     }
+    // tiles that only a caller picks, where the model chooses the chunk alone: as their kin
+    const TileShape& t = kTiles[tile];
+    if (t.kind == 5 || t.kind == 6) return {t.minb, 1.2, t.tx * t.ty / 384.0, 0.8};
+    if (t.kind == 4) return {t.stages, 2.0, l2 ? 0.85 : 1.5, 0.8};
+    return p.precision == 1 ? StepModel{4, 2.0, l2 ? 0.96 : 1.75, 0.8} : StepModel{4, 2.0, l2 ? 1.3 : 1.8, 0.8};
 }
 
 // Time of a step in plane times of the 64x6 tile.
@@ -122,6 +127,11 @@ constexpr int kMaxGridYZ = 65535;
 
 // Whether the tile rows of a lattice fit the second dimension of a grid.
 inline bool rows_fit(int tile, const Plan& p) { return (p.ny + kTiles[tile].ty - 1) / kTiles[tile].ty <= kMaxGridYZ; }
+
+// Whether a launch takes the grid of a tile and z chunk.
+inline bool shape_fits_grid(int tile, int zc, const Plan& p) {
+    return rows_fit(tile, p) && (p.nz + zc - 1) / zc <= kMaxGridYZ;
+}
 
 // Best z chunk of a tile (D3Q19).
 inline int best_zchunk(const Plan& p, int tile, double* cost = nullptr) {
