@@ -169,7 +169,10 @@ typedef struct lbm_sc_handle lbm_sc_handle;
 
 /* Launch shape of the step kernel.  tile selects the CTA tile of x by y
  * columns and the kernel: 0 = 32x8, 1 = 32x16, 2 = 64x8, 3 = 32x4, 4 = 64x4
- * (register-pipelined kernel, every lattice and precision); 5 to 10 are
+ * (register-pipelined kernel, every lattice and precision; tile 3 is the one of an
+ * untuned D2Q9 lattice in 32- and 16-bit storage, where LBM_F32 takes several steps
+ * per launch, and takes 16x8 columns in LBM_F64 on a D3Q19 lattice where those
+ * cover less outside it); 5 to 10 are
  * retired ids (kernels measured slower at every size and removed; rejected
  * with LBM_ERR_INVALID_ARG); 11 = 32x4, 12 = 32x8, 13 = 64x4, 14 = 32x4 (low-register
  * kernel that pulls a plane a second time for its collision, every lattice and
@@ -232,11 +235,13 @@ LBM_SC_API lbm_status lbm_sc_set_stream(lbm_sc_handle* h, void* cuda_stream);
 LBM_SC_API lbm_status lbm_sc_init_fields(lbm_sc_handle* h, const void* d_rhoA, const void* d_rhoB,
                               const void* d_u);
 
-/* Advance nsteps time steps (Eq. eq:be with Eq. FORCE): one fused kernel per
- * step pulls the populations along -c_i (periodic), forms rho_s and j_s, the
+/* Advance nsteps time steps (Eq. eq:be with Eq. FORCE): a fused kernel pulls
+ * the populations along -c_i (periodic), forms rho_s and j_s, the
  * force from the neighbours' densities (plus the body force of Eq. kolmo when
  * body_A != 0), the common velocity u', relaxes each species to
- * f^eq(rho_s, u' + tau_s F_s / rho_s) and stores.  nsteps >= 0. */
+ * f^eq(rho_s, u' + tau_s F_s / rho_s) and stores: one launch per step, or, for
+ * D2Q9 lattices in LBM_F32 on tile 3, two steps per launch (where four or more are
+ * asked for) or all of them in one, with the results of single steps.  nsteps >= 0. */
 LBM_SC_API lbm_status lbm_sc_step(lbm_sc_handle* h, int nsteps);
 
 /* Macroscopic fields of the current state (moments of the populations at the

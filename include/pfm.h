@@ -24,8 +24,11 @@
  * added to the explicit momentum right-hand side (per unit mass; divergence-free).
  * Spectral derivatives: i k for first derivatives (the Nyquist wavenumber of
  * an even axis zeroed), -|k|^2 for the Laplacian; products in physical space,
- * no dealiasing.  Transforms: cuFFT (real-to-complex and back, batched); the
- * spectral and physical-space steps are this library's kernels.
+ * no dealiasing.  Transforms: cuFFT (real-to-complex and back, batched) between
+ * this library's spectral and physical-space kernels; in FP64, on boxes large
+ * enough whose axes are 16 times factors 2, 3, 4, 5 (nx: 32 times), the library's
+ * own transforms inside those kernels.  How a run's steps are divided over calls
+ * does not change their results.
  *
  * Conventions: fields are arrays of nx*ny*nz values, x fastest, in the
  * precision's type (double for PFM_F64, float for PFM_F32); velocities D

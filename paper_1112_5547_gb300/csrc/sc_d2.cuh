@@ -10,10 +10,12 @@
 // runs the second step from there: half the traffic and half the launches for
 // 20 % more collisions (36 x 20 + 32 x 16 for 2 x 512) and 1.6 times the pulls,
 // most of which hit L2.  What bounds it now is the chain of its four phases with
-// two CTAs per SM (45 % of the issue slots used, DRAM at 39 %).  Measured, us a
-// step before and now: 4096^2 461 / 367, 1024^2 34 / 26, 256^2 3.8 / 3.1, eight
-// 256^2 lattices in a batch 20 / 16.6.  Three CTAs of 256 threads that pass every
-// pulled value through shared memory: 352, 26, 3.2, 16.8.
+// two CTAs per SM (DRAM at 48 % of the copy peak at 4096^2).  Measured, us a step
+// before and now: 4096^2 461 / 367, 1024^2 34 / 26, 256^2 3.8 / 3.1, eight 256^2
+// lattices in a batch of 300 steps 19 / 13.7.  Three CTAs of 256 threads that pass
+// every pulled value through shared memory (45 % of the issue slots at 2048^2) take
+// 352, 26 and 3.2, but 434 x 149 3.43 against 3.09: 4 % less at 4096^2 for 11 % more
+// on the middling sizes, so this form serves them all.
 //
 // sc_d2_resident_kernel: all the steps of a call in one launch for a lattice
 // that fits the shared memory of one thread-block cluster.  Each CTA owns a band

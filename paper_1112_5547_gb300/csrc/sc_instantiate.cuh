@@ -25,7 +25,7 @@ cudaError_t step_tiled(const Plan& p, const LatticeArgs<S>& a, cudaStream_t st) 
 
 // Tile 3 in FP64 (D3Q19): 32x4 or 16x8 columns, whichever leaves fewer lanes
 // idle: a warp's FP64 instruction takes its 16 clocks for one active lane as for
-// 32 (48^3, where the second 32-wide tile is half empty: about 125 us a step on 32x4, 98 on 16x8).
+// 32 (48^3, where the second 32-wide tile is half empty: 144 us a step on 32x4, 111 on 16x8).
 template <class L> cudaError_t step_f64_tile3(const Plan& p, const LatticeArgs<double>& a, cudaStream_t st) {
     int tx, ty;
     f64_tile3(p, tx, ty);

@@ -183,8 +183,8 @@ cudaError_t launch_chained(void (*kern)(KA...), dim3 grid, dim3 block, size_t sm
 // fewest, and stay there: where the grid leaves slots free but is larger than the
 // SMs, some SMs then get two or three of them and others none.  Steps of some
 // microseconds gain more from the early launch; the others lose (GB300, us a step,
-// chained / not): FP64 56^3, 168 CTAs 325 / 208; FP64 tile 11 96^3 1006 / 700; FP32
-// tiles 13, 15 and 3 at 96^3 136 / 107, 122 / 91, 96 / 87; but FP32 30^3 - 48^3 10 - 20 % gained.
+// chained / not): FP64 56^3, 168 CTAs 371 / 232; FP64 tile 11 96^3 1172 / 805; FP32
+// tiles 13, 15 and 3 at 96^3 138 / 109, 122 / 91, 96 / 87; but FP32 30^3 - 48^3 10 - 20 % gained.
 // A grid of at most one CTA per SM stays even (FP64 16^3 - 32^3 2 - 8 % gained), and so do
 // the kernels with one CTA per SM and the small CTAs of D2Q9.
 inline bool chain_pays(const Plan& p, dim3 grid) {

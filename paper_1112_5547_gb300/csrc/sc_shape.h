@@ -12,7 +12,7 @@
 // 13: 168 (43), 16: 194 (52), 20: 173 (42), 28: 220 (58), 43: 193 (44 and the
 // one-wave penalty)).  At least 16 planes a chunk on one tile for every lattice,
 // the rule before, gave 313 us there, 18.5 ms instead of 7.1 at 512^3, 84 us
-// instead of 7.4 at 32^3 and 562 instead of 98 at 48^3 in FP64.
+// instead of 7.4 at 32^3 and 562 instead of 111 at 48^3 in FP64.
 #pragma once
 
 #include "sc_launch.cuh"
@@ -49,8 +49,8 @@ inline bool in_l2(const Plan& p) {
 inline StepModel step_model(const Plan& p, int tile) {
     // FP64 is bound by the FP64 units (two FMA a clock and SM): CTAs on one SM
     // share them, density-only planes are nearly free, and one CTA alone leaves
-    // a fifth of the rate unused (48^3 in chunks of 2 / 4 / 6 / 8 planes: 155 /
-    // 144 / 207 / 163 us)
+    // a fifth of the rate unused (48^3 on 32x4 columns in chunks of 2 / 4 / 6 / 8
+    // planes: 154 / 144 / 211 / 159 us)
     if (p.precision == 0) return {1, 0.4, 4.5, 0.8};
     const bool l2 = in_l2(p);
     switch (tile) {
@@ -106,7 +106,7 @@ inline double step_cost(const Plan& p, int tile, int zc) {
     if (p.precision == 0) {
         // CTAs are resident early and share their SM's units: the time is the work
         // of the SM that gets the first CTA of every round (96^3: 24 planes a chunk
-        // 701 us, 20 with a short last chunk 946); one CTA alone on an SM loses a
+        // 803 us, 20 with a short last chunk 1080); one CTA alone on an SM loses a
         // fifth of the rate
         const long long rounds = (full + (last ? xy : 0) + slots - 1) / slots, rfull = (full + slots - 1) / slots;
         end = (double)rfull * a + (double)(rounds - rfull) * b;

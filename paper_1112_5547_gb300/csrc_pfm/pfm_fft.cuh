@@ -14,9 +14,10 @@
 // go in (3 + D fields), and outwards -i k_b (u_a u_b) joins F_a as soon as axis b is
 // transformed (2 + 2 D fields arrive).  The element-wise passes between the
 // transforms are gone, with their divisions.  GB300, ms a step with batched
-// transforms and separate kernels, and so: 512^2 0.467 / 0.327, 128^3 4.83 / 3.26.
+// transforms and separate kernels, and so: 512^2 0.467 / 0.331, 128^3 4.83 / 3.27; small
+// and narrow boxes are faster with batched transforms (fused_pays in pfm.cu).
 // (The FP32 step is bound by memory and instruction issue instead: these kernels in
-// FP32 took 2.8 ms at 256^3 against 2.4, so it keeps the batched transforms.)
+// FP32 took 2.8 ms at 256^3 against 2.2, so it keeps the batched transforms.)
 //
 // Transforms: Stockham autosort in shared memory, radix 4 first and last and any of
 // 2, 3, 4, 5, 8 between, so a length is 16 times a product of those.  In the column

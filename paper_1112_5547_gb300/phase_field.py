@@ -1,7 +1,8 @@
 """Thin ctypes binding of libpfm.so (include/pfm.h): the pseudo-spectral
 phase-field model of Sec. 3 on the GPU.  Argument marshalling only; every step
-runs in the library's kernels and cuFFT.  Raises if the library is missing:
-there is no CPU fallback.
+runs in the library's kernels, with cuFFT between them in FP32 and for the FP64
+boxes that the library's own transforms do not take.  Raises if the library is
+missing: there is no CPU fallback.
 
     from paper_1112_5547_gb300 import phase_field
     s = phase_field.PFM((nz, ny, nx), rho=1.4, tau=0.6, g=0.3, dt=0.1, precision="f32")
